@@ -495,9 +495,9 @@ __global__ void __launch_bounds__(NT) k_schur(const SchurTile* __restrict__ tile
 template <typename T>
 struct ScaleTask {
   const T* B;  // p's row at q's columns, leading dimension ldb
-  const T* Y;  // Y_q, leading dimension nq
+  const T* Y;  // Y_q, leading dimension ldy
   T* O;        // q's row at p's columns, leading dimension ldo
-  int32_t ldb, ldo, np, nq;
+  int32_t ldb, ldo, np, nq, ldy, pad;
 };
 
 template <typename T>
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(NT) k_scale_gemm(const SchurTile* __restrict__
 #pragma unroll
     for (int r = 0; r < NL; ++r) {
       const int e = tid + NT * r, i = e & (TB - 1), k = k0 + e / TB;
-      ry[r] = (i0 + i < d.nq && k < kend) ? d.Y[(i0 + i) + (size_t)k * d.nq] : T(0);
+      ry[r] = (i0 + i < d.nq && k < kend) ? d.Y[(i0 + i) + (size_t)k * d.ldy] : T(0);
       rb[r] = (j0 + i < d.np && k < kend) ? d.B[(j0 + i) + (size_t)k * d.ldb] : T(0);
     }
   };

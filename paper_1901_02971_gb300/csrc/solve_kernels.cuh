@@ -9,6 +9,9 @@
 // T_cf^T r_c followed by the elimination of f, both elimination ops (the
 // first with U = I and X^T = T_cf),
 // and the backward sweep (root -> leaf) the transposes in reverse order.  The
+// OrthS factorization's apply is k_apply_levels (apply_levels.cuh); k_apply
+// below runs the interpolative variants, whose kept dofs are arbitrary
+// subsets of a cluster's (slot lists).  The
 // sparsification transform is kept as the explicit coarse basis Q_pc: since
 // the fine dofs are identity in M^T A M, Q_p [c; f] = r_p + Q_pc (c - c_old)
 // with r_p the forward input, so only Q_pc (|p| x r) and the forward input
@@ -28,9 +31,9 @@ template <typename TF>
 struct ElimOp {
   const TF* XT;      // X^T, ns x m, leading dimension ld >= ns (the right part of s's
                      // block row [U_s | X^T]; T_cf for an interpolation transform)
-  const TF* Y;       // U_s^{-T} (lower, ns x ns, ld = ns); nullptr: U_s = I (the
-                     // interpolation transform T_p of Sec. 2.6.2)
-  int32_t ns, m, ld, pad;
+  const TF* Y;       // U_s^{-T} (lower, ns x ns, leading dimension ldy); nullptr: U_s = I
+                     // (the interpolation transform T_p of Sec. 2.6.2)
+  int32_t ns, m, ld, ldy;
   int64_t slot;      // ns slots of s, then m slots of the neighbour columns
   int64_t ty, tu, ta;  // temp offsets: y_s (ns), u = X_ns y_s (m), backward acc (ns)
 };
@@ -40,12 +43,11 @@ struct ApplyItem {   // one CTA's share of an operation: op index and first row 
 };
 
 template <typename TF>
-struct SqOp {        // scaling S_p followed (if p is sparsified) by Q_p^T, one cluster
-  const TF* Y;       // U_p^{-T} (lower, np x np, ld = np)
-  const TF* Q;       // coarse basis Q_pc (np x r, ld = np); nullptr: not sparsified (r = np)
-  int32_t np, r;
+struct SqOp {        // scaling S_p of one cluster
+  const TF* Y;       // U_p^{-T} (lower, np x np, leading dimension ldy)
+  int32_t np, ldy;
   int64_t slot;      // np slots of p
-  int64_t save;      // np (scaled forward input) + r (coarse values) entries, kept per apply
+  int64_t save;      // np entries: the scaled values, kept per apply
   int64_t tz;        // temp: np entries of the backward sweep
 };
 
@@ -187,8 +189,8 @@ enum ApplyKind : int32_t {
   PH_FU,       //               u = X_ns y_s                  -> tmp[tu]
   PH_SCATTER,  //               x_s = y_s, x_n -= sum u (pull, fixed order)
   PH_SY,       // S_p forward:  y_p = Y x_p                  -> save[0:np]
-  PH_SC,       // Q_p^T:        c = Q_pc^T y_p               -> x (coarse slots), save[np:np+r]
-  PH_SZ,       // Q_p backward: z = y_p + Q_pc (c - c_old)   -> tmp[tz]
+  PH_SC,       //               x_p = y_p
+  PH_SZ,       // S_p backward: z = x_p                      -> tmp[tz]
   PH_SX,       // S_p backward: x_p = Y^T z
   PH_BA,       // E_s backward: acc = x_s - X_ns^T x_n       -> tmp[ta]
   PH_BX        //               x_s = Y^T acc
@@ -219,16 +221,13 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
 // Grid-wide barrier on a monotonically increasing arrival counter (reset to 0
 // before the launch): barrier b completes when the counter reaches
 // (b + 1) * gridDim.x.  All CTAs are co-resident (cooperative launch).  The
-// CTA's writes are ordered before its arrival by bar.sync + a release fence,
-// and the waiter's acquire load + fence order the next phase's reads after
-// every arrival.  The wait is bounded: on timeout *err is set and false is
+// CTA's writes are ordered before its arrival by bar.sync + the release of the
+// arrival, and the waiter's acquire load + fence + bar.sync order the next
+// phase's reads after every arrival.  The wait is bounded: on timeout *err is set and false is
 // returned to every thread of the CTA, which then leaves the kernel.
 __device__ __forceinline__ void grid_arrive(unsigned* count) {
   __syncthreads();
-  if (threadIdx.x == 0) {
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-    asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(count), "r"(1u) : "memory");
-  }
+  if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(count), "r"(1u) : "memory");
 }
 
 __device__ __forceinline__ bool grid_wait(const unsigned* count, unsigned target, int* err, unsigned limit) {
@@ -268,7 +267,7 @@ __device__ __forceinline__ void prefetch_first_item(const ApplyPhase<TF>& P) {
   if (P.kind == PH_FY || P.kind == PH_BA || P.kind == PH_FU || P.kind == PH_BX) {
     const ElimOp<TF> o = P.elim[it.op];
     sl = P.slots + o.slot;
-    ld = (size_t)o.ns;
+    ld = (size_t)o.ldy;
     rows = o.ns;
     if (P.kind == PH_FY) { A = o.Y; rowblock = true; lo = it.first; cols = min(o.ns, it.first + RB); nsl = cols; }
     else if (P.kind == PH_BA) { A = o.XT; ld = (size_t)o.ld; rowblock = true; lo = it.first; cols = o.m; sl += o.ns; nsl = o.m; }
@@ -277,11 +276,10 @@ __device__ __forceinline__ void prefetch_first_item(const ApplyPhase<TF>& P) {
   } else {
     const SqOp<TF> o = P.sq[it.op];
     sl = P.slots + o.slot;
-    ld = (size_t)o.np;
+    ld = (size_t)o.ldy;
     rows = o.np;
     if (P.kind == PH_SY) { A = o.Y; rowblock = true; lo = it.first; cols = min(o.np, it.first + RB); nsl = cols; }
-    else if (P.kind == PH_SZ) { A = o.Q; rowblock = true; lo = it.first; cols = o.Q ? o.r : 0; nsl = o.r; }
-    else if (P.kind == PH_SC) { A = o.Q; rowblock = false; lo = it.first; cols = o.Q ? min(o.r - it.first, AP_COLS) : 0; nsl = 0; }
+    else if (P.kind == PH_SZ || P.kind == PH_SC) { A = nullptr; rowblock = true; lo = it.first; cols = 0; nsl = o.np; }
     else { A = o.Y; rowblock = false; lo = it.first; cols = min(o.np - it.first, AP_COLS); nsl = o.np; }
   }
   for (int k = threadIdx.x * 32; k < nsl; k += AT * 32) prefetch_l2(sl + k);
@@ -342,7 +340,7 @@ __global__ void __launch_bounds__(AT) k_apply(const ApplyPhase<TF>* __restrict__
               if (warp == 0 && i < o.ns) tmp[o.ty + i] = ldv(x + sl[i]);
             } else {
               const int K = min(o.ns, it.first + RB);
-              const ACC v = rowblock_gemv<TF, ACC>(o.Y, (size_t)o.ns, it.first, o.ns, K,
+              const ACC v = rowblock_gemv<TF, ACC>(o.Y, (size_t)o.ldy, it.first, o.ns, K,
                                                    [&](int k) { return ldv(x + sl[k]); }, vs, part);
               if (warp == 0 && i < o.ns) tmp[o.ty + i] = (double)v;
             }
@@ -358,7 +356,7 @@ __global__ void __launch_bounds__(AT) k_apply(const ApplyPhase<TF>* __restrict__
           } else if (!o.Y) {  // PH_BX, U_s = I
             for (int j = it.first + threadIdx.x; j < min(o.ns, it.first + AP_COLS); j += AT) x[sl[j]] = ldv(tmp + o.ta + j);
           } else {  // PH_BX
-            coldot_gemv<TF, ACC>(o.Y, (size_t)o.ns, o.ns, it.first, min(o.ns, it.first + AP_COLS), true,
+            coldot_gemv<TF, ACC>(o.Y, (size_t)o.ldy, o.ns, it.first, min(o.ns, it.first + AP_COLS), true,
                                  [&](int i) { return ldv(tmp + o.ta + i); },
                                  [&](int j, ACC v) { x[sl[j]] = (double)v; }, vs);
           }
@@ -368,37 +366,17 @@ __global__ void __launch_bounds__(AT) k_apply(const ApplyPhase<TF>* __restrict__
           double* sv = save + o.save;
           if (P.kind == PH_SY) {
             const int K = min(o.np, it.first + RB);
-            const ACC v = rowblock_gemv<TF, ACC>(o.Y, (size_t)o.np, it.first, o.np, K,
+            const ACC v = rowblock_gemv<TF, ACC>(o.Y, (size_t)o.ldy, it.first, o.np, K,
                                                  [&](int k) { return ldv(x + sl[k]); }, vs, part);
             const int i = it.first + lane;
             if (warp == 0 && i < o.np) sv[i] = (double)v;
           } else if (P.kind == PH_SC) {
-            const int hi = min(o.r, it.first + AP_COLS);
-            if (o.Q) {
-              coldot_gemv<TF, ACC>(o.Q, (size_t)o.np, o.np, it.first, hi, false, [&](int i) { return ldv(sv + i); },
-                                   [&](int k, ACC c) {
-                                     x[sl[k]] = (double)c;
-                                     sv[o.np + k] = (double)c;
-                                   },
-                                   vs);
-            } else {
-              for (int k = it.first + threadIdx.x; k < hi; k += AT) {
-                const double c = ldv(sv + k);
-                x[sl[k]] = c;
-                sv[o.np + k] = c;
-              }
-            }
+            for (int k = it.first + threadIdx.x; k < min(o.np, it.first + AP_COLS); k += AT) x[sl[k]] = ldv(sv + k);
           } else if (P.kind == PH_SZ) {
             const int i = it.first + lane;
-            if (!o.Q) {
-              if (warp == 0 && i < o.np) tmp[o.tz + i] = ldv(x + sl[i]);
-            } else {
-              const ACC v = rowblock_gemv<TF, ACC>(o.Q, (size_t)o.np, it.first, o.np, o.r,
-                                                   [&](int k) { return ldv(x + sl[k]) - ldv(sv + o.np + k); }, vs, part);
-              if (warp == 0 && i < o.np) tmp[o.tz + i] = ldv(sv + i) + (double)v;
-            }
+            if (warp == 0 && i < o.np) tmp[o.tz + i] = ldv(x + sl[i]);
           } else {  // PH_SX
-            coldot_gemv<TF, ACC>(o.Y, (size_t)o.np, o.np, it.first, min(o.np, it.first + AP_COLS), true,
+            coldot_gemv<TF, ACC>(o.Y, (size_t)o.ldy, o.np, it.first, min(o.np, it.first + AP_COLS), true,
                                  [&](int i) { return ldv(tmp + o.tz + i); },
                                  [&](int j, ACC v) { x[sl[j]] = (double)v; }, vs);
           }

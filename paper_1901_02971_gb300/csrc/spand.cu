@@ -23,6 +23,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "apply_levels.cuh"
 #include "cpqr_cluster.cuh"
 #include "cpqr_reg.cuh"
 #include "factor_kernels.cuh"
@@ -65,6 +66,9 @@ constexpr size_t kCpqrChunkBudget = 224 * 1024;  // shared memory per sparsifica
 constexpr size_t kSmemPerSM = 228 * 1024;        // shared memory of one SM (each resident CTA also reserves 1 KB)
 constexpr int kCpqrMaxCluster = 8;              // thread-block cluster size (broadcasts to 16 CTAs cost 3.5x more)
 constexpr int kAuxStreams = 8;
+constexpr double kCombineWork = 2e9;      // n^2 m of a step's separators up to which their G blocks are formed (FP32)
+constexpr double kApplyStreamBytes = 2e7;  // factor bytes of a phase of the apply from which it is LA_STREAM
+constexpr int64_t kApplyFewItems = 2000;    // 8-row items up to which it is LA_FEW
 constexpr int kApplyCtasPerSm = 4;  // the most CTAs per SM the apply autotuner tries
 
 // Chunked bump allocator over cudaMalloc; reset() keeps the chunks for reuse.
@@ -215,7 +219,6 @@ struct ApplyStep {
   const int32_t* tslot = nullptr;
   const int64_t* tptr = nullptr;
   const int64_t* tidx = nullptr;
-  size_t sm_ns = 0, sm_m = 0, sm_np = 0, sm_r = 0;
   // per-CTA work items of the scaling + coarse-basis GEMVs
   int n_sy = 0, n_sc = 0, n_sz = 0, n_sx = 0;
   const ApplyItem *sy = nullptr, *sc = nullptr, *sz = nullptr, *sx = nullptr;
@@ -505,11 +508,18 @@ struct spand_handle_s {
   // one cooperative launch of k_apply runs it
   const void* aprog = nullptr;
   int n_aprog = 0;
+  // the same for the OrthS variant (apply_levels.cuh)
+  const void* la_phases = nullptr;
+  int n_lphase = 0, la_ctas = 0;
+  DevBuf d_levels;  // the per-level vectors and work areas
+  void* la_vec[8] = {};  // its parts: xh, xl, xs, xsl (nullptr: not needed), y, c, z, u
   int apply_grid = 0;
   int apply_per_sm_max = 1;  // occupancy limit of the apply kernel for this program
   int apply_ctas = 0;        // CTAs per SM of the apply: 0 = not chosen yet (autotuned at the first apply)
   size_t apply_smem = 0;
-  DevBuf d_bar;  // [0] grid-barrier arrival counter, [1] barrier-timeout flag
+  DevBuf d_bar;  // [0] grid-barrier arrival counter, [2] barrier-timeout flag
+  DevBuf d_qc;   // Q_pc of a step's interfaces (written and read on the side stream qs)
+  cudaEvent_t ev_comb = nullptr;  // the last k_combine launch
   unsigned apply_spin_limit = kBarrierSpins;  // polls per grid-barrier wait of the apply
   unsigned apply_bias = 0;                    // 1: failure-path test, no barrier completes
   ~spand_handle_s() {
@@ -518,6 +528,7 @@ struct spand_handle_s {
     if (qs) cudaStreamDestroy(qs);
     if (ev_q) cudaEventDestroy(ev_q);
     if (ev_qdone) cudaEventDestroy(ev_qdone);
+    if (ev_comb) cudaEventDestroy(ev_comb);
     if (ev_fork) cudaEventDestroy(ev_fork);
     for (auto& e : ev_join)
       if (e) cudaEventDestroy(e);
@@ -604,6 +615,7 @@ static void ensure_streams(spand_handle h) {
   CK(cudaStreamCreateWithFlags(&h->qs, cudaStreamNonBlocking));
   CK(cudaEventCreateWithFlags(&h->ev_q, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&h->ev_qdone, cudaEventDisableTiming));
+  CK(cudaEventCreateWithFlags(&h->ev_comb, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
   for (auto& e : h->ev_join) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
 }
@@ -838,16 +850,16 @@ static void add_panels(std::vector<TrsmTask<T>>& out, T* R, const T* dinv, int n
 
 // Y = U^{-T} (lower): the same solve on identity panels (Y must hold I).
 template <typename T>
-static void add_inverse(std::vector<TrsmTask<T>>& out, const T* U, const T* dinv, int n, int ldu, T* Y,
+static void add_inverse(std::vector<TrsmTask<T>>& out, const T* U, const T* dinv, int n, int ldu, T* Y, int ldy,
                         int bw = 0, std::vector<double>* fl = nullptr) {
   for (int c = 0; c < n; c += TB) {
     TrsmTask<T> t;
     t.U = U;
     t.dinv = dinv;
-    t.B = Y + (size_t)c * n;
+    t.B = Y + (size_t)c * ldy;
     t.n = n;
     t.ldu = ldu;
-    t.ldb = n;
+    t.ldb = ldy;
     t.nc = std::min(c + TB, n) - c;
     t.i_start = c;
     t.bw = bw;
@@ -1423,7 +1435,7 @@ static std::vector<InterpOut<T>> sparsify_interp(spand_handle h, const std::vect
         diag.push_back({F, nf, d.ldf, dv, 0, 0});
         fcls[c].push_back(d.p);
         add_panels(tr, F, (const T*)dv, nf, d.ldf, nf, d.np);
-        add_inverse(tr, (const T*)F, (const T*)dv, nf, d.ldf, Yf);
+        add_inverse(tr, (const T*)F, (const T*)dv, nf, d.ldf, Yf, nf);
         if (r > 0) {
           const int np = d.np;
           double* Tt = d.G;
@@ -1595,6 +1607,7 @@ static ApplyStep<T> make_elim_step(spand_handle h, const std::vector<ElimSpec<T>
     o.Y = sp.Y;
     o.ld = sp.ld;
     o.ns = (int32_t)sp.s_slots.size();
+    o.ldy = o.ns;
     o.m = (int32_t)sp.n_slots.size();
     if (o.ns == 0) continue;
     o.slot = (int64_t)aslots.size();
@@ -1648,6 +1661,284 @@ static ApplyStep<T> make_elim_step(spand_handle h, const std::vector<ElimSpec<T>
   ap.ba = at<const ApplyItem>(d, oba);
   ap.bx = at<const ApplyItem>(d, obx);
   return ap;
+}
+
+// Apply of the OrthS factorization (apply_levels.cuh): the operations of every
+// step, uploaded as the steps are factorized, and the running sizes of the
+// work vectors.
+template <typename T>
+struct LevelProgram {
+  struct Step {
+    const LevelOp<T>*e = nullptr, *s = nullptr;
+    const int64_t* list = nullptr;
+    const int32_t* base[8] = {};  // per phase kind: first item of every operation
+    int nitems[8] = {};
+    int ne = 0, ns = 0;
+    bool combined = false;  // the separators' G blocks are formed
+    int emode = LA_MID, smode = LA_MID;  // LevelMode of the E and S phases
+  };
+  std::vector<Step> steps;
+  int64_t xs = 0, xs_next = 0;  // places of X_t and X_{t+1}
+  int64_t y = 0, c = 0, u = 0, z = 0;
+  bool pass = false;  // some clusters are not scaled: their values pass through
+};
+
+// Forms G_ns or P_p (k_combine) on the side stream, after everything issued on
+// s so far; the sparsification of a later step, and the end of the
+// factorization, wait for ev_comb.
+template <typename T>
+static void combine_batch(spand_handle h, const std::vector<CombineTask<T>>& tasks, cudaStream_t s) {
+  std::vector<CombineTile> tiles;
+  for (size_t k = 0; k < tasks.size(); ++k)
+    for (int j0 = 0; j0 < tasks[k].n; j0 += TB)
+      for (int i0 = 0; i0 < tasks[k].m; i0 += TB) tiles.push_back({(int32_t)k, i0, j0});
+  if (tiles.empty()) return;
+  ensure_streams(h);
+  Packer pk;
+  const size_t ot = pk.add(tiles), ok = pk.add(tasks);
+  void* d = upload<T>(h, pk, s);
+  CK(cudaEventRecord(h->ev_q, s));
+  CK(cudaStreamWaitEvent(h->qs, h->ev_q, 0));
+  k_combine<T><<<(unsigned)tiles.size(), NT, 0, h->qs>>>(at<const CombineTile>(d, ot), at<const CombineTask<T>>(d, ok));
+  CKLAUNCH();
+  h->prof.launches += 1;
+  CK(cudaEventRecord(h->ev_comb, h->qs));
+}
+
+// Adds step t's operations (its sizes and ranks are known).  pof / ro: the
+// remaining clusters' parents and row offsets in them (nullptr at the root);
+// nsz: sizes of step t + 1; gfac: the separators' G blocks (empty: two-phase
+// form); pfac: the interfaces' P blocks (nullptr: not sparsified).
+template <typename T>
+static void add_level_step(spand_handle h, LevelProgram<T>& lp, int t, const std::vector<int>& seps,
+                           const std::vector<int>& rems, const Layout<T>& lay, const std::vector<int32_t>& sz,
+                           const std::vector<int32_t>& sz_after, const std::vector<T*>& ysep,
+                           const std::vector<T*>& gfac, const std::vector<SqOp<T>>& sqops,
+                           const std::vector<int>& sq_cluster, const std::vector<T*>& pfac,
+                           const std::vector<int32_t>* pof, const std::vector<int32_t>* ro,
+                           const std::vector<int32_t>& nsz, cudaStream_t s) {
+  const int n = (int)sz.size();
+  auto al4 = [](int64_t v) { return (v + 3) & ~int64_t(3); };
+  std::vector<int64_t> xbase(n + 1, 0), nbase;
+  const int64_t x0 = t == 1 ? 0 : lp.xs;
+  for (int i = 0; i < n; ++i) xbase[i + 1] = xbase[i] + sz[i];
+  if (pof) {
+    nbase.assign(nsz.size() + 1, lp.xs_next);
+    for (size_t i = 0; i < nsz.size(); ++i) nbase[i + 1] = nbase[i] + nsz[i];
+  }
+  typename LevelProgram<T>::Step st;
+  st.combined = !gfac.empty();
+  {  // LA_STREAM by bytes; LA_FEW by the 8-row items of the forward phases, where those take several rounds of loads
+    const int round = 64 * LaGeom<T>::VW / 2;  // columns that 8 loads of an 8-row item cover
+    double eb = 0, sb = 0;
+    int64_t ei = 0, si = 0;
+    int32_t en = 0, sn = 0;
+    for (int i : seps) {
+      const double m = lay.W[i] - sz[i];
+      eb += ((double)sz[i] * sz[i] / 2 + sz[i] * m) * sizeof(T);
+      ei += (sz[i] + 7) / 8 + (st.combined ? ((int)m + 7) / 8 : 0);
+      en = std::max(en, sz[i]);
+    }
+    for (int i : rems) {
+      sb += ((double)sz[i] * sz[i] / 2 + (double)sz[i] * sz_after[i]) * sizeof(T);
+      si += (sz[i] + 7) / 8 + (sz_after[i] + 7) / 8;
+      sn = std::max(sn, sz[i]);
+    }
+    auto mode = [&](double bytes, int64_t items, int32_t nmax) {
+      return bytes >= kApplyStreamBytes ? LA_STREAM : items <= kApplyFewItems && nmax > round ? LA_FEW : LA_MID;
+    };
+    st.emode = mode(eb, ei, en);
+    st.smode = mode(sb, si, sn);
+  }
+  std::vector<LevelOp<T>> e, sp;
+  std::vector<int32_t> base[8];
+  auto count = [&](int kind, const LevelOp<T>& o) {
+    base[kind].push_back(st.nitems[kind]);
+    st.nitems[kind] += la_items<T>(kind, o.n, o.m, o.A != nullptr, o.Y != nullptr,
+                                   kind == LP_FS || kind == LP_BS ? st.smode : st.emode);
+  };
+  std::vector<int32_t> np(n + 1, 0);  // pieces per remaining cluster
+  int64_t u = 0, z = 0, tmp_off = 0;
+  for (int i : seps) {
+    if (sz[i] <= 0) continue;
+    LevelOp<T> o{};
+    o.n = sz[i];
+    o.m = lay.W[i] - sz[i];
+    o.ldy = row_ld(sz[i]);
+    o.Y = ysep[i];
+    if (st.combined) {
+      o.lda = row_ld(o.m);
+      o.A = gfac[i];
+    } else {
+      o.lda = lay.ld[i];
+      o.A = lay.row[i] + (size_t)lay.ld[i] * sz[i];
+      o.z = z;
+      z += al4(o.n);
+    }
+    o.x = x0 + xbase[i];
+    o.y = lp.y;
+    lp.y += al4(o.n);
+    o.u = u;
+    for (int32_t k = lay.nptr[i]; k < lay.nptr[i + 1]; ++k)
+      if (sz[lay.nidx[k]] > 0) ++np[lay.nidx[k] + 1];
+    u += al4(o.m);
+    h->st.mem_f += (int64_t)o.n * (o.n + 1) / 2 + (int64_t)o.n * o.m;
+    tmp_off += 2 * (int64_t)o.n + o.m;
+    if (st.combined) count(LP_FE, o), count(LP_BE, o);
+    else count(LP_FY, o), count(LP_FU, o), count(LP_BA, o), count(LP_BX, o);
+    e.push_back(o);
+  }
+  lp.u = std::max(lp.u, u);
+  lp.z = std::max(lp.z, z);
+  for (int i = 0; i < n; ++i) np[i + 1] += np[i];
+  std::vector<int64_t> list(np[n]);
+  {
+    std::vector<int32_t> at(np.begin(), np.end() - 1);
+    size_t k = 0;
+    for (int i : seps) {
+      if (sz[i] <= 0) continue;
+      for (int32_t q = lay.nptr[i]; q < lay.nptr[i + 1]; ++q)
+        if (sz[lay.nidx[q]] > 0) list[at[lay.nidx[q]]++] = e[k].u + (lay.noff[q] - sz[i]);
+      ++k;
+    }
+  }
+  if (pof) {
+    std::vector<int> sq_of(n, -1);
+    for (size_t i = 0; i < sq_cluster.size(); ++i) sq_of[sq_cluster[i]] = (int)i;
+    for (int i : rems) {
+      if (sz[i] <= 0) continue;
+      LevelOp<T> o{};
+      o.n = sz[i];
+      o.m = sz_after[i];
+      o.lda = row_ld(o.m);
+      o.ldy = row_ld(o.n);
+      o.A = pfac[i];
+      o.Y = sq_of[i] >= 0 ? sqops[sq_of[i]].Y : nullptr;
+      if (!o.Y) lp.pass = true;
+      o.x = x0 + xbase[i];
+      o.u = nbase[(*pof)[i]] + (*ro)[i];
+      o.l0 = np[i];
+      o.nl = np[i + 1] - np[i];
+      if (o.Y) {
+        o.y = lp.y;
+        lp.y += al4(o.n);
+        h->save_len += (int64_t)o.n + o.m;
+        tmp_off += o.n;
+      }
+      if (o.A) {
+        o.c = lp.c;
+        lp.c += al4(o.m);
+      }
+      count(LP_FS, o), count(LP_BS, o);
+      sp.push_back(o);
+    }
+    lp.xs = lp.xs_next;
+    lp.xs_next = nbase.back();
+  }
+  h->tmp_len = std::max(h->tmp_len, tmp_off);
+  Packer pk;
+  const size_t oe = pk.add(e), os = pk.add(sp), ol = pk.add(list);
+  size_t ob[8];
+  for (int k = 0; k < 8; ++k) ob[k] = pk.add(base[k]);
+  if (!pk.empty()) {
+    void* d = h->persist.alloc(pk.size);
+    void* src = h->stage.take(pk.size);
+    pk.write(src);
+    CK(cudaMemcpyAsync(d, src, pk.size, cudaMemcpyHostToDevice, s));
+    st.e = at<const LevelOp<T>>(d, oe);
+    st.s = at<const LevelOp<T>>(d, os);
+    st.list = at<const int64_t>(d, ol);
+    for (int k = 0; k < 8; ++k) st.base[k] = at<const int32_t>(d, ob[k]);
+  }
+  st.ne = (int)e.size();
+  st.ns = (int)sp.size();
+  lp.steps.push_back(std::move(st));
+}
+
+// Phases per launch at most (their descriptors take 72 KB of shared memory, three CTAs per SM).
+constexpr int kLevelMaxPhases = 96;
+
+// The phases in execution order and the items of each.
+template <typename T>
+static void finish_level_program(spand_handle h, const LevelProgram<T>& lp, cudaStream_t s) {
+  const int L = (int)lp.steps.size();
+  std::vector<LevelPhase<T>> ph;
+  size_t nitems = 0;
+  auto add = [&](int kind, int t) {
+    const auto& st = lp.steps[t];
+    const bool sq = kind == LP_FS || kind == LP_BS;
+    LevelPhase<T> p{};
+    p.kind = kind;
+    p.ops = sq ? st.s : st.e;
+    p.nops = sq ? st.ns : st.ne;
+    p.list = st.list;
+    p.base = st.base[kind];
+    p.nitems = st.nitems[kind];
+    p.first = t == 0;
+    p.mode = sq ? st.smode : st.emode;
+    if (p.nitems <= 0) return;
+    nitems += (size_t)p.nitems;
+    ph.push_back(p);
+  };
+  auto down = [&](int t) {
+    if (lp.steps[t].combined) add(LP_FE, t);
+    else add(LP_FY, t), add(LP_FU, t);
+    add(LP_FS, t);
+  };
+  auto back = [&](int t) {
+    add(LP_BS, t);
+    if (lp.steps[t].combined) add(LP_BE, t);
+    else add(LP_BA, t), add(LP_BX, t);
+  };
+  for (int t = 0; t < L; ++t) down(t);
+  for (int t = L - 1; t >= 0; --t) back(t);
+  h->n_lphase = (int)ph.size();
+  h->n_aprog = 0;
+  const int np = h->n_lphase;
+  const void* fn = (const void*)k_apply_levels<T>;
+  const size_t smem = la_smem<T>(std::min(np, kLevelMaxPhases));
+  ensure_smem(fn, smem + 1024);  // the kernel's static shared memory counts too
+  int per_sm = 0;
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, LA_NT, smem));
+  if (per_sm < 1) throw Fail{SPAND_ERR_CUDA, "apply kernel cannot be resident"};
+  h->apply_per_sm_max = std::min(per_sm, kApplyCtasPerSm);
+  h->apply_grid = num_sms() * (h->apply_ctas > 0 ? std::min(h->apply_ctas, h->apply_per_sm_max) : h->apply_per_sm_max);
+  LevelItem* items = (LevelItem*)h->persist.alloc(nitems * sizeof(LevelItem));
+  int maxops = 1;
+  for (LevelPhase<T>& p : ph) {
+    p.items = items;
+    items += p.nitems;
+    maxops = std::max(maxops, p.nops);
+  }
+  // no more CTAs than the phase of most items has work for
+  int most = 1;
+  for (const LevelPhase<T>& p : ph) most = std::max(most, p.nitems);
+  h->la_ctas = (most + LA_NW - 1) / LA_NW;
+  if (np) {
+    Packer pk;
+    const size_t op = pk.add(ph);
+    void* d = h->persist.alloc(pk.size);
+    void* src = h->stage.take(pk.size);
+    pk.write(src);
+    CK(cudaMemcpyAsync(d, src, pk.size, cudaMemcpyHostToDevice, s));
+    h->la_phases = at<const LevelPhase<T>>(d, op);
+    k_level_items<T><<<dim3((unsigned)std::min((maxops + 127) / 128, 256), (unsigned)np), 128, 0, s>>>(
+        (const LevelPhase<T>*)h->la_phases);
+    CKLAUNCH();
+    h->prof.launches += 1;
+  }
+  h->d_bar.ensure(3 * sizeof(unsigned));
+  CK(cudaMemsetAsync(h->d_bar.p, 0, 3 * sizeof(unsigned), s));
+  auto al4 = [](int64_t v) { return (v + 3) & ~int64_t(3); };
+  const int64_t n1 = sizeof(T) == 4 ? al4(h->n) : 0, xs = al4(lp.xs_next), lo = sizeof(T) == 4 && lp.pass ? xs : 0;
+  const int64_t len[8] = {n1, n1, xs, lo, al4(lp.y), al4(lp.c), al4(lp.z), al4(lp.u)};
+  int64_t tot = 0;
+  for (int64_t l : len) tot += l;
+  T* w = (T*)h->d_levels.ensure((size_t)std::max<int64_t>(tot, 1) * sizeof(T));
+  for (int k = 0; k < 8; ++k) {
+    h->la_vec[k] = len[k] || k > 3 ? w : nullptr;
+    w += len[k];
+  }
 }
 
 // The apply program: the phases of every step in execution order (forward
@@ -1707,8 +1998,9 @@ static void build_apply_program(spand_handle h, const std::vector<ApplyStep<TF>>
     CK(cudaMemcpyAsync(d, src, ph.size() * sizeof(ApplyPhase<TF>), cudaMemcpyHostToDevice, s));
     h->aprog = d;
   }
-  h->d_bar.ensure(2 * sizeof(unsigned));
-  CK(cudaMemsetAsync(h->d_bar.p, 0, 2 * sizeof(unsigned), s));
+  h->n_lphase = 0;
+  h->d_bar.ensure(3 * sizeof(unsigned));
+  CK(cudaMemsetAsync(h->d_bar.p, 0, 3 * sizeof(unsigned), s));
   const void* fn = (const void*)k_apply<TF>;
   h->apply_smem = (size_t)SCH * sizeof(TF) + ph.size() * sizeof(ApplyPhase<TF>);
   ensure_smem(fn, h->apply_smem);
@@ -1786,9 +2078,12 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
   std::vector<std::vector<int32_t>> slots(nc0);
   for (int i = 0; i < nc0; ++i) {
     sz[i] = tr.cluster_ptr[i + 1] - tr.cluster_ptr[i];
+    if (h->opts.variant == SPAND_ORTHS) continue;  // its apply needs no slot lists
     slots[i].resize(sz[i]);
     std::iota(slots[i].begin(), slots[i].end(), tr.cluster_ptr[i]);
   }
+  const bool levels = h->opts.variant == SPAND_ORTHS;  // the apply works on per-level vectors (apply_levels.cuh)
+  LevelProgram<T> lp;
   CK(cudaEventRecord(tm.at(0, 0), s));
   Layout<T> lay = make_layout<T>(h, 1, sz, s);
   {  // assemble A into the step-1 rows
@@ -1848,10 +2143,11 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         diag_fl.push_back(cfl);
         add_panels(tr_tasks, lay.row[sidx], (const T*)dv, sz[sidx], lay.ld[sidx], sz[sidx], lay.W[sidx], bw, &tr_fl,
                    nnzU);
-        T* Y = (T*)h->persist.alloc((size_t)sz[sidx] * sz[sidx] * sizeof(T));
+        const int ldy = row_ld(sz[sidx]);
+        T* Y = (T*)h->persist.alloc((size_t)ldy * sz[sidx] * sizeof(T));
         ysep[sidx] = Y;
-        ident.push_back({Y, sz[sidx], sz[sidx], nullptr, 0, 0});
-        add_inverse(tr_tasks, (const T*)lay.row[sidx], (const T*)dv, sz[sidx], lay.ld[sidx], Y, bw, &tr_fl);
+        ident.push_back({Y, sz[sidx], ldy, nullptr, 0, 0});
+        add_inverse(tr_tasks, (const T*)lay.row[sidx], (const T*)dv, sz[sidx], lay.ld[sidx], Y, ldy, bw, &tr_fl);
         stt.factor_flops += cfl + 2 * nnzU * m + ns * m * m;
       }
       set_identity<T>(h, ident, s);
@@ -2027,6 +2323,24 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
     }
     CK(cudaEventRecord(tm.at(t, 1), s));
     // ------------------------------------------------ apply ops of the elimination
+    std::vector<T*> gfac;  // per separator: G_ns = X_ns Y_s (empty: the two-phase form)
+    if (levels) {
+      double work = 0;
+      for (int i : seps) work += (double)sz[i] * sz[i] * (lay.W[i] - sz[i]);
+      if (work <= kCombineWork / (sizeof(T) == 8 ? 20 : 1)) {
+        gfac.assign(n, nullptr);
+        std::vector<CombineTask<T>> gt;
+        for (int i : seps) {
+          const int m = lay.W[i] - sz[i];
+          if (sz[i] <= 0) continue;
+          const int ldg = row_ld(m);
+          gfac[i] = (T*)h->persist.alloc((size_t)ldg * sz[i] * sizeof(T));
+          if (m > 0)
+            gt.push_back({lay.row[i] + (size_t)lay.ld[i] * sz[i], ysep[i], gfac[i], sz[i], m, lay.ld[i], row_ld(sz[i]), ldg, 0});
+        }
+        combine_batch<T>(h, gt, s);
+      }
+    }
     ApplyStep<T> ap;
     std::vector<int32_t> aslots = h->pool32.take();
     std::vector<ElimOp<T>> eops;
@@ -2037,11 +2351,12 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
     std::vector<ApplyItem> it_fy = h->poolitem.take(), it_fu = h->poolitem.take(), it_ba = h->poolitem.take(),
                            it_bx = h->poolitem.take();
     int64_t tmp_off = 0;
-    size_t sm_ns = 0, sm_m = 0;
     int64_t nassign = 0;
     bool elim_ops_built = false;
     // built after the sparsification launches (its host time then overlaps them)
     auto build_elim_ops = [&]() {
+      elim_ops_built = true;
+      if (levels) return;
       for (int sidx : seps) {
         if (sz[sidx] <= 0) continue;
         ElimOp<T> o{};
@@ -2049,6 +2364,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         o.ld = lay.ld[sidx];
         o.Y = ysep[sidx];
         o.ns = sz[sidx];
+        o.ldy = row_ld(o.ns);
         o.m = lay.W[sidx] - sz[sidx];
         o.slot = (int64_t)aslots.size();
         o.ty = tmp_off;
@@ -2078,14 +2394,11 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         tmp_off += 2 * (int64_t)o.ns + o.m;
         eops.push_back(o);
         stt.mem_f += (int64_t)o.ns * (o.ns + 1) / 2 + (int64_t)o.ns * o.m;
-        sm_ns = std::max(sm_ns, (size_t)o.ns * sizeof(double));
-        sm_m = std::max(sm_m, (size_t)o.m * sizeof(double));
       }
       h->tmp_len = std::max(h->tmp_len, tmp_off);
       nassign = (int64_t)tslot.size();
       group_by_target(h, h->n, tgt, tslot, tptr, tidx);
       h->poolpair.give(std::move(tgt));
-      elim_ops_built = true;
     };
 
     // ------------------------------------------------ scale + sparsify
@@ -2094,7 +2407,6 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
     std::vector<SqOp<T>> sqops;
     std::vector<int> sq_cluster;
     std::vector<int> cp_index;  // per cluster: index in cp_cluster, -1 if not sparsified
-    size_t sm_np = 0, sm_r = 0;
     const bool sparsify = (skip < t) && (t < L);
     int cpqr_pid = -1;
     std::vector<int> ell_fin;              // randomized compression: final sketch width per task
@@ -2104,6 +2416,8 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
     std::vector<ApplyStep<T>> interp_steps;  // their apply groups: T_p ops, then the eliminations of f
     std::vector<int> cp_cluster;           // sparsified clusters (task order)
     std::vector<T*> cp_qc;                 // their Q_pc scratch
+    std::vector<T*> ypin(n, nullptr);       // per scaled cluster: its pivot inverse
+    std::vector<T*> pfac(n, nullptr);       // per cluster: P_p in the factor (nullptr: not sparsified)
     if (sparsify) {
       std::vector<RowDesc<T>> diag, ident;
       std::vector<int> diag_cl;
@@ -2140,21 +2454,21 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           b.cols = sz[q];
           m_lo.push_back(b);
         }
-        T* Y = (T*)h->persist.alloc((size_t)sz[p] * sz[p] * sizeof(T));
-        ident.push_back({Y, sz[p], sz[p], nullptr});
-        add_inverse(up, (const T*)lay.row[p], (const T*)dv, sz[p], lay.ld[p], Y);
+        const int ldy = row_ld(sz[p]);
+        T* Y = (T*)h->persist.alloc((size_t)ldy * sz[p] * sizeof(T));
+        ident.push_back({Y, sz[p], ldy, nullptr});
+        add_inverse(up, (const T*)lay.row[p], (const T*)dv, sz[p], lay.ld[p], Y, ldy);
         idr.push_back({lay.row[p], sz[p], lay.ld[p], nullptr});
         SqOp<T> so{};
         so.Y = Y;
-        so.Q = nullptr;
         so.np = sz[p];
-        so.r = sz[p];
+        so.ldy = ldy;
+        ypin[p] = Y;
         sqops.push_back(so);
         sq_cluster.push_back(p);
         const double np_ = sz[p], m = lay.W[p] - sz[p];
         stt.factor_flops += np_ * np_ * np_ / 3 + np_ * np_ * m;
         stt.mem_f += (int64_t)sz[p] * (sz[p] + 1) / 2;
-        sm_np = std::max(sm_np, (size_t)sz[p] * sizeof(double));
       }
       // second side of every pair p < q from the first side's block and Y_q:
       // O = Y_q (U_p^{-T} A_pq)^T into q's row (the scaled A_qp)
@@ -2172,6 +2486,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           k.np = c.cols;
           k.nq = c.rows;
           k.Y = nullptr;
+          k.ldy = row_ld(c.rows);
           sct.push_back(k);
         }
         size_t i = 0;
@@ -2231,7 +2546,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       std::vector<int> tres;    // 1: the task's chunk lives in shared memory
       std::vector<int> treg;    // lane-group size of the register-resident kernel (0: chunked kernel)
       const int ncol = st.ncolours();
-      size_t wbytes = 0;
+      size_t wbytes = 0, qbytes = 0;
       struct WOff { size_t nrm, v, tau, qc, gw; };
       std::vector<WOff> woff;
       const size_t CB = kCpqrChunkBudget;
@@ -2283,7 +2598,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         w.nrm = 0;
         w.v = wbytes; wbytes += align256((size_t)sz[p] * sz[p] * sizeof(T));
         w.tau = wbytes; wbytes += align256((size_t)sz[p] * sizeof(T));
-        w.qc = wbytes; wbytes += align256((size_t)sz[p] * sz[p] * sizeof(T));
+        w.qc = qbytes; qbytes += align256((size_t)sz[p] * sz[p] * sizeof(T));
         w.gw = wbytes;
         if (!resident && !interp) wbytes += align256((size_t)C * Lp * ((mm + C - 1) / C) * sizeof(T));
         woff.push_back(w);
@@ -2347,10 +2662,12 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       }
       if (!tasks.empty()) {
         char* wb = interp ? nullptr : (char*)h->scratch[(t + 1) & 1].ensure(wbytes);
+        char* qb = interp ? nullptr : (char*)h->d_qc.ensure(qbytes);
+        if (h->ev_comb) CK(cudaStreamWaitEvent(s, h->ev_comb, 0));  // the previous step's Q_pc have been read
         for (size_t i = 0; i < tasks.size() && wb; ++i) {
           tasks[i].V = (T*)(wb + woff[i].v);
           tasks[i].tau = (T*)(wb + woff[i].tau);
-          tasks[i].Qc = (T*)(wb + woff[i].qc);
+          tasks[i].Qc = (T*)(qb + woff[i].qc);
           tasks[i].gwork = (T*)(wb + woff[i].gw);
           cp_qc.push_back(tasks[i].Qc);
         }
@@ -2583,19 +2900,16 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         }
       }
       for (int sidx : seps) sz_after[sidx] = 0;
-      // compact Q_pc (|p| x r) into the factor
-      std::vector<CopyTask<T>> qcopy;
-      std::vector<int> sq_of(n, -1);
-      for (size_t i = 0; i < sq_cluster.size(); ++i) sq_of[sq_cluster[i]] = (int)i;
+      // P_p = Q_pc^T Y_p (r x |p|) into the factor
+      std::vector<CombineTask<T>> ptasks;
       for (size_t i = 0; i < cp_cluster.size() && !interp; ++i) {
         const int p = cp_cluster[i];
         const int r = sz_after[p];
-        // sparsified: Q_pc (|p| x r); r = 0 keeps a non-null empty basis
-        T* Q = (T*)h->persist.alloc((size_t)sz[p] * std::max(r, 1) * sizeof(T));
-        if (r > 0) qcopy.push_back({cp_qc[i], Q, sz[p], sz[p], sz[p], r, 0, 0});
-        SqOp<T>& so = sqops[sq_of[p]];
-        so.Q = Q;
-        so.r = r;
+        // sparsified: r = 0 keeps a non-null empty block
+        const int ldp_ = row_ld(r);
+        T* P = (T*)h->persist.alloc((size_t)ldp_ * sz[p] * sizeof(T));
+        pfac[p] = P;
+        if (r > 0) ptasks.push_back({cp_qc[i], ypin[p], P, sz[p], r, sz[p], row_ld(sz[p]), ldp_, 0});
         const double np_ = sz[p], m = lay.W[p] - sz[p], rr = r;
         // CPQR of A_pn to rank r; randomized: sketch and projection (2 np m ell
         // each) and the QR of the np x ell sketch
@@ -2607,8 +2921,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         h->prof.add(cpqr_pid, qfl, (np_ * m + 2 * rr * m + np_ * rr) * sizeof(T));
         stt.mem_f += (int64_t)sz[p] * r;
       }
-      for (auto& so : sqops) sm_r = std::max(sm_r, (size_t)std::max(so.r, 1) * sizeof(double));
-      copy_batch<T>(h, qcopy, s);
+      combine_batch<T>(h, ptasks, s);
       if (interp) {
         // apply groups of the step's interpolative transforms: T_p (U = I,
         // X^T = T_cf, c against f), then the elimination of f against c; p
@@ -2649,6 +2962,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           pof[a] = P;
           ro[a] = o;
           o += sz_after[a];
+          if (levels) continue;
           const std::vector<int32_t>& ks = has_kept[a] ? kept_slots[a] : slots[a];
           nslots[P].insert(nslots[P].end(), ks.begin(), ks.begin() + sz_after[a]);
         }
@@ -2703,13 +3017,21 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         }
       }
       copy_batch<T>(h, cps, s);
+      if (levels)
+        add_level_step<T>(h, lp, t, seps, rems, lay, sz, sz_after, ysep, gfac, sqops, sq_cluster, pfac, &pof, &ro, nsz, s);
       sz = nsz;
       slots_of_step = std::move(slots);
       slots = std::move(nslots);
     } else {
+      if (levels)
+        add_level_step<T>(h, lp, t, seps, rems, lay, sz, sz_after, ysep, gfac, sqops, sq_cluster, pfac, nullptr, nullptr, sz, s);
       slots_of_step = std::move(slots);
     }
     CK(cudaEventRecord(tm.at(t, 4), s));
+    if (levels) {
+      if (t < L) lay = std::move(nxt);
+      continue;
+    }
     run_pending();  // the previous step's program, if the GPU never waited for us
     // The step's apply program (scaling + coarse-basis ops, upload) is built
     // later, during the next step's sparsification kernels (run_pending), so
@@ -2720,8 +3042,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       pending = [h, s, &apply, prev_slots = std::move(prev_slots), ap = std::move(ap), eops = std::move(eops),
                  sqops = std::move(sqops), sq_cluster = std::move(sq_cluster), aslots = std::move(aslots),
                  tslot = std::move(tslot), tptr = std::move(tptr), tidx = std::move(tidx), it_fy = std::move(it_fy),
-                 it_fu = std::move(it_fu), it_ba = std::move(it_ba), it_bx = std::move(it_bx), nassign, sm_ns, sm_m,
-                 sm_np, sm_r, tmp_off, interp_steps = std::move(interp_steps)]() mutable {
+                 it_fu = std::move(it_fu), it_ba = std::move(it_ba), it_bx = std::move(it_bx), nassign, tmp_off, interp_steps = std::move(interp_steps)]() mutable {
       // slots, save areas, temporaries and work items of the scaling +
       // coarse-basis ops (step-t slot lists)
       std::vector<ApplyItem> it_sy = h->poolitem.take(), it_sc = h->poolitem.take(), it_sz = h->poolitem.take(),
@@ -2734,7 +3055,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           so.slot = (int64_t)aslots.size();
           aslots.insert(aslots.end(), prev_slots[p].begin(), prev_slots[p].end());
           so.save = save;
-          save += so.np + so.r;
+          save += 2 * (int64_t)so.np;
           so.tz = tmp_off;
           tmp_off += so.np;
           const int32_t op = (int32_t)i;
@@ -2742,7 +3063,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
             it_sy.push_back({op, r0});
             it_sz.push_back({op, r0});
           }
-          for (int32_t c0 = 0; c0 < so.r; c0 += AP_COLS) it_sc.push_back({op, c0});
+          for (int32_t c0 = 0; c0 < so.np; c0 += AP_COLS) it_sc.push_back({op, c0});
           for (int32_t c0 = 0; c0 < so.np; c0 += AP_COLS) it_sx.push_back({op, c0});
         }
         h->save_len = save;
@@ -2787,10 +3108,6 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         ap.fu = at<const ApplyItem>(d, ofu);
         ap.ba = at<const ApplyItem>(d, oba);
         ap.bx = at<const ApplyItem>(d, obx);
-        ap.sm_ns = sm_ns;
-        ap.sm_m = sm_m;
-        ap.sm_np = sm_np;
-        ap.sm_r = sm_r;
         apply.push_back(ap);
         for (const ApplyStep<T>& x : interp_steps)
           if (x.n_elim) apply.push_back(x);
@@ -2807,6 +3124,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
     if (t < L) lay = std::move(nxt);
   }
   run_pending();
+  if (h->ev_comb) CK(cudaStreamWaitEvent(s, h->ev_comb, 0));
   CK(cudaStreamSynchronize(s));
   check_pivots(L);
   {
@@ -2818,6 +3136,10 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         CK(cudaEventElapsedTime(&ms, tm.at(t, k), tm.at(t, k + 1)));
         h->phase_ms[k] += ms;
       }
+  }
+  if (levels) {
+    finish_level_program<T>(h, lp, s);
+    return SPAND_OK;
   }
   build_apply_program<T>(h, apply, s);
   if constexpr (std::is_same<T, double>::value) {
@@ -2832,16 +3154,70 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
 
 // ---------------------------------------------------------------- apply / PCG
 
+// The level program: one cooperative launch (several for very deep
+// dissections).
+template <typename TF>
+static int launch_levels(spand_handle h, const LevelVecs<TF>& V, cudaStream_t s) {
+  int nl = 0;
+  for (int p0 = 0; p0 < h->n_lphase; p0 += kLevelMaxPhases, ++nl) {
+    const LevelPhase<TF>* ph = (const LevelPhase<TF>*)h->la_phases + p0;
+    int np = std::min(kLevelMaxPhases, h->n_lphase - p0);
+    unsigned lim = h->apply_spin_limit, bias = h->apply_bias;
+    unsigned* bar = (unsigned*)h->d_bar.p;
+    int* err = (int*)h->d_bar.p + 2;
+    LevelVecs<TF> v = V;
+    CK(cudaMemsetAsync(bar, 0, sizeof(unsigned), s));
+    void* args[] = {(void*)&ph, (void*)&np, (void*)&v, (void*)&bar, (void*)&err, (void*)&lim, (void*)&bias};
+    CK(cudaLaunchCooperativeKernel((const void*)k_apply_levels<TF>, dim3((unsigned)std::min(h->apply_grid, h->la_ctas)),
+                                   dim3(LA_NT), args, la_smem<TF>(np), s));
+    CKLAUNCH();
+  }
+  h->prof.launches += nl;
+  return nl;
+}
+
+template <typename TF>
+static void apply_levels(spand_handle h, const double* src, double* dst, cudaStream_t s) {
+  const int pid = h->prof.begin(F_APPLY, s);
+  LevelVecs<TF> v{};
+  TF** part[8] = {nullptr, nullptr, &v.xs, &v.xsl, &v.y, &v.c, &v.z, &v.u};
+  for (int k = 2; k < 8; ++k) *part[k] = (TF*)h->la_vec[k];
+  v.out = dst;
+  int nl = 0;
+  if constexpr (std::is_same<TF, double>::value) {
+    v.xh = src;
+  } else {
+    v.xh = (const TF*)h->la_vec[0];
+    v.xl = (const TF*)h->la_vec[1];
+    k_split<<<(unsigned)std::min<int64_t>((h->n + 255) / 256, 4096), 256, 0, s>>>(h->n, src, (float*)h->la_vec[0],
+                                                                                 (float*)h->la_vec[1]);
+    CKLAUNCH();
+    h->prof.launches += 1;
+    nl = 1;
+  }
+  nl += launch_levels<TF>(h, v, s);
+  h->prof.end(pid, s, 0.0, h->st.apply_bytes, nl);
+}
+
 // tmp: h->tmp_len doubles of per-step temporaries; save: h->save_len doubles
 // of sparsification forward inputs (both scratch; nothing needs to start at 0).
 // One cooperative launch runs the whole apply program; a barrier timeout is
-// recorded in d_bar[1] and reported by check_apply().
+// recorded in d_bar[2] and reported by check_apply().
 template <typename TF>
-static void apply_prec(spand_handle h, double* x, double* tmp, double* save, cudaStream_t s) {
+static void apply_prec(spand_handle h, const double* src, double* x, double* tmp, double* save, cudaStream_t s) {
+  if (h->n_lphase) {
+    apply_levels<TF>(h, src, x, s);
+    return;
+  }
+  if (src != x) {
+    k_copy_vec<<<(unsigned)std::min<int64_t>((h->n + 255) / 256, 4096), 256, 0, s>>>(h->n, src, x);
+    CKLAUNCH();
+    h->prof.launches += 1;
+  }
   if (!h->n_aprog) return;
   const int pid = h->prof.begin(F_APPLY, s);
   unsigned* bar = (unsigned*)h->d_bar.p;
-  int* err = (int*)(bar + 1);
+  int* err = (int*)(bar + 2);
   CK(cudaMemsetAsync(bar, 0, sizeof(unsigned), s));
   const ApplyPhase<TF>* ph = (const ApplyPhase<TF>*)h->aprog;
   int nph = h->n_aprog;
@@ -2855,9 +3231,10 @@ static void apply_prec(spand_handle h, double* x, double* tmp, double* save, cud
   h->prof.end(pid, s, 0.0, h->st.apply_bytes, 1);
 }
 
-static void apply_any(spand_handle h, double* x, double* tmp, double* save, cudaStream_t s) {
-  if (h->fprec == SPAND_FP64) apply_prec<double>(h, x, tmp, save, s);
-  else apply_prec<float>(h, x, tmp, save, s);
+// dst = M M^T src (in cluster order; the two may be the same vector).
+static void apply_any(spand_handle h, const double* src, double* dst, double* tmp, double* save, cudaStream_t s) {
+  if (h->fprec == SPAND_FP64) apply_prec<double>(h, src, dst, tmp, save, s);
+  else apply_prec<float>(h, src, dst, tmp, save, s);
 }
 
 // Reads (after the stream has been synchronised) and clears the apply's
@@ -2865,15 +3242,15 @@ static void apply_any(spand_handle h, double* x, double* tmp, double* save, cuda
 static void check_apply(spand_handle h) {
   if (!h->d_bar.p) return;
   int flag = 0;
-  CK(cudaMemcpy(&flag, (unsigned*)h->d_bar.p + 1, sizeof(int), cudaMemcpyDeviceToHost));
+  CK(cudaMemcpy(&flag, (unsigned*)h->d_bar.p + 2, sizeof(int), cudaMemcpyDeviceToHost));
   if (flag) {
-    CK(cudaMemset((unsigned*)h->d_bar.p + 1, 0, sizeof(int)));
+    CK(cudaMemset((unsigned*)h->d_bar.p + 2, 0, sizeof(int)));
     throw Fail{SPAND_ERR_TIMEOUT, "preconditioner apply: a grid barrier timed out"};
   }
 }
 
-static void apply_any(spand_handle h, double* x, cudaStream_t s) {
-  apply_any(h, x, (double*)h->d_tmp.p, (double*)h->d_save.p, s);
+static void apply_any(spand_handle h, const double* src, double* dst, cudaStream_t s) {
+  apply_any(h, src, dst, (double*)h->d_tmp.p, (double*)h->d_save.p, s);
 }
 
 // Tile-shape autotuner of the apply (the grid of its cooperative launch):
@@ -2884,7 +3261,7 @@ static void apply_any(spand_handle h, double* x, cudaStream_t s) {
 // changes a bit of z.  More CTAs stream the large leaf phases faster; fewer
 // make the grid barriers of many small phases cheaper.
 static void apply_autotune(spand_handle h, double* scratch, cudaStream_t s) {
-  if (h->apply_ctas > 0 || !h->n_aprog) return;
+  if (h->apply_ctas > 0 || !(h->n_aprog || h->n_lphase)) return;
   int nsm = 0, dev = 0;
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -2898,10 +3275,10 @@ static void apply_autotune(spand_handle h, double* scratch, cudaStream_t s) {
   int pick = h->apply_per_sm_max;
   for (int c = 1; c <= h->apply_per_sm_max; ++c) {
     h->apply_grid = nsm * c;
-    apply_any(h, scratch, s);  // warm-up
+    apply_any(h, scratch, scratch, s);  // warm-up
     CK(cudaEventRecord(e0, s));
-    apply_any(h, scratch, s);
-    apply_any(h, scratch, s);
+    apply_any(h, scratch, scratch, s);
+    apply_any(h, scratch, scratch, s);
     CK(cudaEventRecord(e1, s));
     CK(cudaEventSynchronize(e1));
     float ms = 0.f;
@@ -3238,7 +3615,7 @@ int spand_apply(spand_handle h, const double* r_dev, double* z_dev, void* cuda_s
   const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, 4096);
   k_permute<<<g, 256, 0, s>>>(n, (const int32_t*)h->d_perm.p, r_dev, w, 1);
   CKLAUNCH();
-  apply_any(h, w, s);
+  apply_any(h, w, w, s);
   k_permute<<<g, 256, 0, s>>>(n, (const int32_t*)h->d_perm.p, w, z_dev, 0);
   CKLAUNCH();
   h->prof.launches += 2;
@@ -3302,7 +3679,7 @@ int spand_apply_noalloc(spand_handle h, const double* r_dev, double* z_dev, void
   const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, 4096);
   k_permute<<<g, 256, 0, s>>>(n, (const int32_t*)h->d_perm.p, r_dev, w, 1);
   CKLAUNCH();
-  apply_any(h, w, tmp, save, s);
+  apply_any(h, w, w, tmp, save, s);
   k_permute<<<g, 256, 0, s>>>(n, (const int32_t*)h->d_perm.p, w, z_dev, 0);
   CKLAUNCH();
   h->prof.launches += 2;
@@ -3365,11 +3742,8 @@ int spand_solve(spand_handle h, const double* b, double* x, int32_t* iters, doub
   double apply_ms = 0, spmv_ms = 0;
   int napply = 0;
   auto precond = [&](const double* src, double* dst) {
-    k_copy_vec<<<g, 256, 0, s>>>(n, src, dst);
-    CKLAUNCH();
-    h->prof.launches += 1;
     CK(cudaEventRecord(e0, s));
-    apply_any(h, dst, s);
+    apply_any(h, src, dst, s);
     CK(cudaEventRecord(e1, s));
     CK(cudaEventSynchronize(e1));
     float ms = 0;

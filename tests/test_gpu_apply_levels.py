@@ -1,0 +1,43 @@
+"""The preconditioner apply (spand_apply) on sizes at the edges of its work items.
+
+With eps = 0 nothing is compressed and M M^T = A^{-1}, so z is compared with a
+sparse direct solve.  Tolerance, fixed beforehand: the explicit inverse factors
+and the products carry rounding errors of a small multiple of cond(A) u
+(u = 2^-53 or 2^-24, the factor's unit roundoff); 20 cond(A) u is allowed, with
+cond(A) of the grid Laplacian from its known eigenvalues."""
+import numpy as np
+import pytest
+import scipy.sparse.linalg as sla
+
+from paper_1901_02971_gb300 import Solver
+from paper_1901_02971_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+# (dimension, grid side, levels): a root of 25 unknowns alone; one taller than
+# a round of loads; leaves of a few hundred odd-sized rows; leaves beyond 512
+# rows; many small clusters that pass through unscaled; a root whose factor is
+# large enough for the streaming cut of its items in FP32 (4096 rows) and FP64
+CASES = [(2, 5, 1), (2, 31, 1), (3, 9, 2), (3, 12, 2), (2, 33, 6), (3, 17, 6), (3, 16, 1)]
+
+
+def _cond(dim, n):
+    lam = [2 - 2 * np.cos(k * np.pi / (n + 1)) for k in (1, n)]
+    return lam[1] / lam[0]  # the dimensions add equally
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("dim,n,levels", CASES)
+def test_exact_apply_is_the_inverse(cuda_ok, dim, n, levels, precision):
+    import torch
+    p = I.laplacian_2d(n) if dim == 2 else I.laplacian_3d(n)
+    r = I.rhs(p.n, 3)
+    ref = sla.spsolve(p.to_scipy().tocsc(), r)
+    s = Solver.from_problem(p, levels=levels, eps=0.0, precision=precision).factorize()
+    try:
+        z = s.apply(torch.from_numpy(r).cuda()).cpu().numpy()
+    finally:
+        s.close()
+    u = 2.0 ** (-53 if precision == "fp64" else -24)
+    err = np.linalg.norm(z - ref) / np.linalg.norm(ref)
+    assert err <= 20 * _cond(dim, n) * u, err
