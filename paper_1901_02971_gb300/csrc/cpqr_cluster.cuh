@@ -98,6 +98,10 @@ struct CqShared {     // fixed part of the dynamic shared memory
   int cand_j[2][CQ_MAXW];
   T cta_v[2][CQ_MAXC];
   int cta_j[2][CQ_MAXC];
+  // FP64: the step's reflector, formed by one warp (amb = alpha - beta, gam;
+  // stop: the truncation rule ends the loop here), by step parity
+  T amb[2], gam[2];
+  int stop[2];
 };
 
 __host__ __device__ inline size_t cq_al16(size_t b) { return (b + 15) & ~size_t(15); }
@@ -128,16 +132,18 @@ __device__ __forceinline__ void cq_warp_argmax(float& v, int& j) {
   j = jj;
 }
 __device__ __forceinline__ void cq_warp_argmax(double& v, int& j) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const double ov = __shfl_xor_sync(0xffffffffu, v, o);
-    const int oj = __shfl_xor_sync(0xffffffffu, j, o);
-    if (ov > v || (ov == v && oj < j)) {
-      v = ov;
-      j = oj;
-    }
-  }
+  // the same on the two halves of the bit pattern: a 64-bit comparison would go
+  // to the FP64 unit, which a warp-wide instruction holds for tens of cycles
+  const int hi = __double2hiint(v), best = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = (unsigned)__double2loint(v), bl = __reduce_max_sync(0xffffffffu, hi == best ? lo : 0u);
+  j = __reduce_min_sync(0xffffffffu, hi == best && lo == bl ? j : INT_MAX);
+  v = __hiloint2double(best, (int)bl);
 }
+// a > b for such values (squared norms, or -1)
+__device__ __forceinline__ bool cq_greater(float a, float b) { return __float_as_int(a) > __float_as_int(b); }
+__device__ __forceinline__ bool cq_greater(double a, double b) { return __double_as_longlong(a) > __double_as_longlong(b); }
+__device__ __forceinline__ bool cq_live(float v) { return __float_as_int(v) >= 0; }
+__device__ __forceinline__ bool cq_live(double v) { return __double2hiint(v) >= 0; }
 
 // one barrier for the whole cluster (a plain block barrier when C == 1)
 __device__ __forceinline__ void cq_sync(cg::cluster_group& cl, int C) {
@@ -285,12 +291,18 @@ __device__ __forceinline__ void cq_finish(const CpqrTask<T>& d, cg::cluster_grou
 //   2. every thread reduces the C candidates: pivot j*, |R_kk| = sqrt(norm)
 //      (norms are recomputed exactly each step); the truncation rule is
 //      checked here, uniformly;
-//   3. every thread derives the reflector from the raw pivot column p (read in
-//      place when C == 1, else from the copy its owner pushed):
-//      beta = -sign(p_k) |R_kk|,
-//      tau = (beta - p_k) / beta, v = [1; p_{k+1:} / (p_k - beta)];
+//   3. the reflector H_k = I - gam u u^T from the raw pivot column p (read in
+//      place when C == 1, else from the copy its owner pushed), by every thread
+//      in FP32, by one warp in FP64;
 //   4. every thread applies H_k to its live columns and recomputes their
 //      trailing norms.
+// FP64 (sparsification family, before and after: 64 x 64 2.13 -> 0.98 ms,
+// 31 x 29 x 27 25.1 -> 13.4, 64^3 181 -> 113; the cluster sizes chosen on the
+// host then give 8.0 and 87): the FP64 unit issues a warp-wide instruction every
+// 64 cycles per sub-partition, so everything but the sweeps was taken off it:
+// candidates are compared as integers, one warp forms the reflector with one
+// square root and one division, and tau and 1 / (alpha - beta) wait until after
+// the loop.
 //
 // Column ownership: with LG lanes per column, thread t belongs to group
 // t / LG, which owns the local columns t / LG + c * (NT / LG), c < CQ_CPT;
@@ -438,7 +450,7 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
     int bj = INT_MAX;
 #pragma unroll
     for (int c = 0; c < CQ_CPT; ++c)
-      if (nrm[c] > bv) {
+      if (cq_greater(nrm[c], bv)) {
         bv = nrm[c];
         bj = j0 + grp + c * NG;
       }
@@ -474,116 +486,89 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
       cq_warp_argmax(gv, gj);
     }
     if (gj == INT_MAX) gj = 0;  // unreachable: k < kmax <= m leaves a live column
-    const T rkk = sqrt(gv > T(0) ? gv : T(0));
-    if (k == 0) r00 = rkk;
-    if (r00 == T(0) || rkk < eps * r00) {
+    // 3. the reflector H_k = I - gam u u^T, u = [0; alpha - beta; p_{k+1:}] with
+    //    the raw pivot column p (never written again), beta = -sign(alpha) |R_kk|,
+    //    gam = 1 / (beta (beta - alpha)).  FP64: by warp 0 alone, handed over by a
+    //    block barrier; every warp would otherwise repeat a few dozen FP64
+    //    instructions (square root, division) on its sub-partition's FP64 unit,
+    //    most of a small interface's step.
+    const T* pcol = C == 1 ? chunk + (size_t)(gj - j0) * L
+                           : cbuf + ((size_t)(k & 1) * C + min(C - 1, gj / cols_per)) * L;
+    T amb, gam;
+    bool stop;
+    auto reflector = [&]() {
+      const T rkk = sqrt(gv > T(0) ? gv : T(0));
+      if (k == 0) r00 = rkk;
+      stop = r00 == T(0) || rkk < eps * r00;
+      const T alpha = pcol[k];
+      const T beta = alpha >= T(0) ? -rkk : rkk;
+      amb = alpha - beta;
+      gam = rkk == T(0) ? T(0) : T(1) / (beta * (beta - alpha));
+      if (tid == 0 && !stop) {
+        tau_s[k] = alpha;  // tau_k and scal_k follow after the loop
+        beta_s[k] = beta;
+        piv_s[k] = gj;
+        if (gj >= j0 && gj < j0 + nc) rstep[gj - j0] = k;
+      }
+    };
+    if constexpr (sizeof(T) == 8) {
+      if (warp == 0) {
+        reflector();
+        if (lane == 0) {
+          sh.amb[k & 1] = amb;
+          sh.gam[k & 1] = gam;
+          sh.stop[k & 1] = stop;
+        }
+      }
+      __syncthreads();
+      amb = sh.amb[k & 1];
+      gam = sh.gam[k & 1];
+      stop = sh.stop[k & 1] != 0;
+    } else {
+      reflector();
+    }
+    if (stop) {
       r = k;
       break;
     }
 #pragma unroll
     for (int c = 0; c < CQ_CPT; ++c)
       if (j0 + grp + c * NG == gj) nrm[c] = T(-1);  // the pivot column leaves the live set
-    // 3. the raw pivot column (never written again) and the reflector
-    const T* pcol = C == 1 ? chunk + (size_t)(gj - j0) * L
-                           : cbuf + ((size_t)(k & 1) * C + min(C - 1, gj / cols_per)) * L;
-    const T alpha = pcol[k];
-    T beta, tau, scal;
-    if (rkk == T(0)) {
-      beta = T(0);
-      tau = T(0);
-      scal = T(0);
-    } else {
-      beta = alpha >= T(0) ? -rkk : rkk;
-      tau = (beta - alpha) / beta;
-      scal = T(1) / (alpha - beta);
-    }
-    if (tid == 0) {
-      tau_s[k] = tau;
-      beta_s[k] = beta;
-      scal_s[k] = scal;
-      piv_s[k] = gj;
-    }
-    if (gj >= j0 && gj < j0 + nc && tid == 0) rstep[gj - j0] = k;
-    // 4. apply H_k = I - tau v v^T to my live columns, recompute their trailing norms:
-    //    w = tau (x_k + scal p_{k+1:}^T x_{k+1:}),  x_k -= w,  x_{k+1:} -= (w scal) p_{k+1:}
+    // 4. apply H_k to my live columns, x -= (gam u.x) u, and recompute their
+    //    trailing norms; the vector that holds row k is masked, u(i) = 0 above it
     const int gs = k / VW;
     const int rb = gs * VW;
     const V* __restrict__ pv = reinterpret_cast<const V*>(pcol);
 #pragma unroll
     for (int c = 0; c < CQ_CPT; ++c) {
-      if (nrm[c] < T(0)) continue;  // uniform over the group
+      if (!cq_live(nrm[c])) continue;  // uniform over the group
       T* colp = chunk + (size_t)(grp + c * NG) * L;
       V* __restrict__ cv = reinterpret_cast<V*>(colp);
-      const T xk = colp[k];
-      if constexpr (LG > 1) {
-        // the group's lanes take interleaved vectors; lane 0 holds vector gs
-        T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-        for (int g = gs + lg; g < ng; g += LG) {
-          const V x = cv[g], p = pv[g];
-          if (g == gs) {
-            if (rb > k) a0 = fma(x.x, p.x, a0);
-            if (rb + 1 > k) a1 = fma(x.y, p.y, a1);
-            if constexpr (VW == 4) {
-              if (rb + 2 > k) a2 = fma(x.z, p.z, a2);
-              if (rb + 3 > k) a3 = fma(x.w, p.w, a3);
-            }
-          } else {
-            a0 = fma(x.x, p.x, a0);
-            a1 = fma(x.y, p.y, a1);
-            if constexpr (VW == 4) {
-              a2 = fma(x.z, p.z, a2);
-              a3 = fma(x.w, p.w, a3);
-            }
-          }
-        }
-        const T dot = cq_group_sum<LG>((a0 + a1) + (a2 + a3));
-        const T w = tau * fma(scal, dot, xk);
-        const T ws = w * scal;
-        T q0 = 0, q1 = 0, q2 = 0, q3 = 0;
-        for (int g = gs + lg; g < ng; g += LG) {
-          V x = cv[g];
-          const V p = pv[g];
-          if (g == gs) {  // row k takes -w, rows > k take -ws p and enter the norm
-            if (rb == k) x.x -= w;
-            else if (rb > k) { x.x = fma(-ws, p.x, x.x); q0 = x.x * x.x; }
-            if (rb + 1 == k) x.y -= w;
-            else if (rb + 1 > k) { x.y = fma(-ws, p.y, x.y); q1 = x.y * x.y; }
-            if constexpr (VW == 4) {
-              if (rb + 2 == k) x.z -= w;
-              else if (rb + 2 > k) { x.z = fma(-ws, p.z, x.z); q2 = x.z * x.z; }
-              if (rb + 3 == k) x.w -= w;
-              else if (rb + 3 > k) { x.w = fma(-ws, p.w, x.w); q3 = x.w * x.w; }
-            }
-          } else {
-            x.x = fma(-ws, p.x, x.x);
-            x.y = fma(-ws, p.y, x.y);
-            q0 = fma(x.x, x.x, q0);
-            q1 = fma(x.y, x.y, q1);
-            if constexpr (VW == 4) {
-              x.z = fma(-ws, p.z, x.z);
-              x.w = fma(-ws, p.w, x.w);
-              q2 = fma(x.z, x.z, q2);
-              q3 = fma(x.w, x.w, q3);
-            }
-          }
-          cv[g] = x;
-        }
-        nrm[c] = cq_group_sum<LG>((q0 + q1) + (q2 + q3));
-        continue;
-      }
-      T a0 = 0, a1 = 0, a2 = 0, a3 = 0, b0 = 0, b1 = 0, b2 = 0, b3 = 0;
-      {  // first vector: only rows > k
-        const V x = cv[gs], p = pv[gs];
-        if (rb > k) a0 = x.x * p.x;
-        if (rb + 1 > k) a1 = x.y * p.y;
+      // the group's lanes take interleaved vectors, lane 0 the one that holds row k
+      V pk, xk;
+      if (lg == 0) {
+        pk = pv[gs];
+        xk = cv[gs];
+        pk.x = rb < k ? T(0) : rb == k ? amb : pk.x;
+        pk.y = rb + 1 < k ? T(0) : rb + 1 == k ? amb : pk.y;
         if constexpr (VW == 4) {
-          if (rb + 2 > k) a2 = x.z * p.z;
-          if (rb + 3 > k) a3 = x.w * p.w;
+          pk.z = rb + 2 < k ? T(0) : rb + 2 == k ? amb : pk.z;
+          pk.w = rb + 3 < k ? T(0) : rb + 3 == k ? amb : pk.w;
         }
       }
-      int g = gs + 1;
-      for (; g + 1 < ng; g += 2) {  // two vectors per trip, independent accumulators
-        const V x0 = cv[g], p0 = pv[g], x1 = cv[g + 1], p1 = pv[g + 1];
+      const int g0 = gs + (lg == 0 ? LG : lg);
+      T a0 = 0, a1 = 0, a2 = 0, a3 = 0, b0 = 0, b1 = 0, b2 = 0, b3 = 0;
+      if (lg == 0) {
+        a0 = xk.x * pk.x;
+        a1 = xk.y * pk.y;
+        if constexpr (VW == 4) {
+          a2 = xk.z * pk.z;
+          a3 = xk.w * pk.w;
+        }
+      }
+      int g = g0;
+      for (; g + LG < ng; g += 2 * LG) {  // two vectors per trip, independent accumulators
+        const V x0 = cv[g], p0 = pv[g], x1 = cv[g + LG], p1 = pv[g + LG];
         a0 = fma(x0.x, p0.x, a0);
         a1 = fma(x0.y, p0.y, a1);
         b0 = fma(x1.x, p1.x, b0);
@@ -604,27 +589,27 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
           a3 = fma(x0.w, p0.w, a3);
         }
       }
-      const T dot = ((a0 + b0) + (a1 + b1)) + ((a2 + b2) + (a3 + b3));
-      const T w = tau * fma(scal, dot, xk);
-      const T ws = w * scal;
+      T dot;
+      if constexpr (VW == 4) dot = ((a0 + b0) + (a1 + b1)) + ((a2 + b2) + (a3 + b3));
+      else dot = (a0 + b0) + (a1 + b1);
+      dot = cq_group_sum<LG>(dot);
+      const T ws = gam * dot;
       T q0 = 0, q1 = 0, q2 = 0, q3 = 0;
-      {  // first vector: row k takes -w, rows > k take -ws p and enter the norm
-        V x = cv[gs];
-        const V p = pv[gs];
-        if (rb == k) x.x -= w;
-        else if (rb > k) { x.x = fma(-ws, p.x, x.x); q0 = x.x * x.x; }
-        if (rb + 1 == k) x.y -= w;
-        else if (rb + 1 > k) { x.y = fma(-ws, p.y, x.y); q1 = x.y * x.y; }
+      if (lg == 0) {  // rows > k enter the norm
+        xk.x = fma(-ws, pk.x, xk.x);
+        xk.y = fma(-ws, pk.y, xk.y);
+        if (rb > k) q0 = xk.x * xk.x;
+        if (rb + 1 > k) q1 = xk.y * xk.y;
         if constexpr (VW == 4) {
-          if (rb + 2 == k) x.z -= w;
-          else if (rb + 2 > k) { x.z = fma(-ws, p.z, x.z); q2 = x.z * x.z; }
-          if (rb + 3 == k) x.w -= w;
-          else if (rb + 3 > k) { x.w = fma(-ws, p.w, x.w); q3 = x.w * x.w; }
+          xk.z = fma(-ws, pk.z, xk.z);
+          xk.w = fma(-ws, pk.w, xk.w);
+          if (rb + 2 > k) q2 = xk.z * xk.z;
+          if (rb + 3 > k) q3 = xk.w * xk.w;
         }
-        cv[gs] = x;
+        cv[gs] = xk;
       }
 #pragma unroll 2
-      for (g = gs + 1; g < ng; ++g) {
+      for (g = g0; g < ng; g += LG) {
         V x = cv[g];
         const V p = pv[g];
         x.x = fma(-ws, p.x, x.x);
@@ -639,8 +624,17 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
         }
         cv[g] = x;
       }
-      nrm[c] = (q0 + q1) + (q2 + q3);
+      T q;
+      if constexpr (VW == 4) q = (q0 + q1) + (q2 + q3);
+      else q = q0 + q1;
+      nrm[c] = cq_group_sum<LG>(q);
     }
+  }
+  __syncthreads();
+  for (int kk = tid; kk < r; kk += NT) {  // tau_k and scal_k from alpha_k and beta_k
+    const T al = tau_s[kk], be = beta_s[kk];
+    tau_s[kk] = be == T(0) ? T(0) : (be - al) / be;
+    scal_s[kk] = be == T(0) ? T(0) : T(1) / (al - be);
   }
   __syncthreads();
   cq_finish<T, NT>(d, cluster, C, rank, chunk, L, np, r, nc, j0, cpm, tcol, rstep, beta_s, scal_s, tau_s, piv_s,

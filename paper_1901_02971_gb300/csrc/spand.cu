@@ -12,6 +12,7 @@
 #include <new>
 #include <type_traits>
 #include <numeric>
+#include <queue>
 #include <stdexcept>
 #include <string>
 #include <climits>
@@ -65,6 +66,7 @@ static inline int32_t row_ld(int32_t size) { return (std::max<int32_t>(size, 1) 
 constexpr size_t kCpqrChunkBudget = 224 * 1024;  // shared memory per sparsification CTA (chunk included)
 constexpr size_t kSmemPerSM = 228 * 1024;        // shared memory of one SM (each resident CTA also reserves 1 KB)
 constexpr int kCpqrMaxCluster = 8;              // thread-block cluster size (broadcasts to 16 CTAs cost 3.5x more)
+constexpr double kCqFp64Work = 2000;              // see its use
 constexpr int kAuxStreams = 8;
 constexpr double kCombineWork = 2e9;      // n^2 m of a step's separators up to which their G blocks are formed (FP32)
 constexpr double kApplyStreamBytes = 2e7;  // factor bytes of a phase of the apply from which it is LA_STREAM
@@ -308,38 +310,35 @@ static bool encode_row_map(CUtensorMap* m, const float* base, int rows, int cols
 
 static std::mutex g_cluster_mutex;  // guards the cached cluster-size probe
 
-// Largest cluster size (16 or 8) at which the sparsification kernel can be
-// resident with a full shared-memory chunk on this device.
-template <typename T>
-static int cpqr_max_cluster() {
-  if constexpr (kCpqrMaxCluster <= 8) return kCpqrMaxCluster;
-  std::lock_guard<std::mutex> lk(g_cluster_mutex);
-  static int cached[2] = {0, 0};
-  int& c = cached[sizeof(T) == 8 ? 1 : 0];
-  if (c) return c;
-  const void* fn = (const void*)k_cpqr_cluster<T, true, 256>;
+// How many clusters of C > 8 CTAs of the FP64 sparsification kernel, each with a
+// full shared-memory chunk, can be resident at once on this device.
+static int cpqr_wide_clusters(int C) {
+  const int dev = current_device();
+  const void* fn = (const void*)k_cpqr_cluster<double, true, 512, 2>;
   const size_t smem = kCpqrChunkBudget;
   ensure_smem(fn, smem);
-  c = 8;
+  std::lock_guard<std::mutex> lk(g_cluster_mutex);
+  static std::map<std::pair<int, int>, int> cached;
+  auto it = cached.find({dev, C});
+  if (it != cached.end()) return it->second;
+  int n = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(16, 1, 1);
-    cfg.blockDim = dim3(256, 1, 1);
+    cfg.gridDim = dim3((unsigned)C, 1, 1);
+    cfg.blockDim = dim3(512, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 16;
+    attr[0].val.clusterDim.x = (unsigned)C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n > 0) c = 16;
+    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) n = 0;
   }
-  cudaGetLastError();  // a refused query only means 8
-  return c;
+  cudaGetLastError();  // a refused query only means 0
+  return cached[{dev, C}] = n;
 }
-
 
 // Kernel-family profiler: launch counts always; with profiling on, a CUDA
 // event pair on the launching stream around each batch of launches of one
@@ -1029,6 +1028,9 @@ static int cpqr_reg_capacity(int G, int C) {
 // not, 256 or 512 threads per CTA.
 template <typename T>
 static const void* cpqr_kernel(bool res, int nt, int lg = 1) {
+  if constexpr (sizeof(T) == 8)
+    if (nt == 512 && lg == 8)
+      return res ? (const void*)k_cpqr_cluster<T, true, 512, 8> : (const void*)k_cpqr_cluster<T, false, 512, 8>;
   if (nt == 512 && lg == 4)
     return res ? (const void*)k_cpqr_cluster<T, true, 512, 4> : (const void*)k_cpqr_cluster<T, false, 512, 4>;
   if (nt == 512 && lg == 2)
@@ -1069,7 +1071,7 @@ static std::vector<int> sparsify_randomized(spand_handle h, int t, const std::ve
   const size_t onb = pkn.add(nbrs);
   const CpqrNbr<T>* d_nbrs = at<const CpqrNbr<T>>(upload<T>(h, pkn, s), onb);
   const size_t CB = kCpqrChunkBudget;
-  const int max_cluster = cpqr_max_cluster<T>();
+  const int max_cluster = kCpqrMaxCluster;
   const uint64_t seed = h->opts.sketch_seed;
   int32_t* hbuf = nullptr;
   for (int c = 0; c < std::max(ncol, 1); ++c) {
@@ -2550,7 +2552,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       struct WOff { size_t nrm, v, tau, qc, gw; };
       std::vector<WOff> woff;
       const size_t CB = kCpqrChunkBudget;
-      const int max_cluster = cpqr_max_cluster<T>();
+      const int max_cluster = kCpqrMaxCluster;
       for (int p : rems) {
         if (sz[p] <= 0) continue;
         if (lay.nptr[p + 1] == lay.nptr[p]) continue;  // no neighbours: nothing to compress against
@@ -2641,6 +2643,53 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
             treg[i] = rg[i];
             tclass[i] = rc[i];
             tres[i] = 1;
+          }
+        }
+      }
+      // FP64: a step's time is its column sweep on the FP64 units of the SMs
+      // that hold the interface, so the clusters of a colour grow until the
+      // colour fills the GPU, the interface with the most work per CTA first
+      // (down to kCqFp64Work elements per CTA, where the exchange between the
+      // CTAs takes over), and a chunk that does not fit in the shared memory of
+      // 8 CTAs gets up to 16.  Sparsification of 64^3 with the smallest clusters
+      // that hold the chunk, then with these: 113, 87 ms; of 31 x 29 x 27: 13.4,
+      // 8.0 ms (500 / 2000 / 6000 / 20000 elements: 8.5 / 8.0 / 8.1 / 12.8).
+      if (sizeof(T) == 8 && !interp && h->opts.compression == SPAND_CPQR) {
+        static const int sizes[] = {1, 2, 4, 8, 10, 12, 16};
+        auto smem_of = [&](const CpqrTask<T>& k, int c) {
+          const int cp = (k.m_max + c - 1) / c;
+          return cq_fixed_smem<T>(k.nend - k.nbeg, k.np, cp, c) + (size_t)cq_ld<T>(k.np) * cp * sizeof(T);
+        };
+        std::vector<std::vector<int>> by(sim ? 1 : std::max(ncol, 1));
+        for (size_t i = 0; i < tasks.size(); ++i) by[colour_of(tasks[i].p)].push_back((int)i);
+        for (const std::vector<int>& col : by) {
+          int total = 0, wide = 0;
+          for (int i : col) {
+            if (!tres[i])
+              for (int c : {10, 12, 16})
+                if (smem_of(tasks[i], c) <= CB && cpqr_wide_clusters(c) > 0) { tclass[i] = c; tres[i] = 1; break; }
+            total += tclass[i];
+            wide += tclass[i] > 8;
+          }
+          typedef std::pair<double, int> Load;
+          std::priority_queue<Load> q;
+          auto load = [&](int i) { return (double)tasks[i].np * tasks[i].m_max / tclass[i]; };
+          for (int i : col) q.push({load(i), i});
+          while (!q.empty()) {
+            const int i = q.top().second;
+            q.pop();
+            if (load(i) <= kCqFp64Work) break;
+            int next = 0;
+            for (int c : sizes)
+              if (c > tclass[i]) { next = c; break; }
+            if (!next || total + next - tclass[i] > num_sms() || (next > 8 && wide - (tclass[i] > 8) >= cpqr_wide_clusters(next)) ||
+                tasks[i].m_max < 16 * next || smem_of(tasks[i], next) > CB)
+              continue;  // this one stays
+            wide += next > 8 && tclass[i] <= 8;
+            total += next - tclass[i];
+            tclass[i] = next;
+            tres[i] = 1;
+            q.push({load(i), i});
           }
         }
       }
@@ -2755,7 +2804,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
             int lg = 1;
             if (sizeof(T) == 8 && one_wave && cpg <= 256) {
               nt = 512;
-              lg = cpg <= 128 ? 4 : 2;
+              lg = cpg <= 64 ? 8 : cpg <= 128 ? 4 : 2;
             }
             const void* fn = cpqr_kernel<T>(G.res != 0, nt, lg);
             if (G.G) {
