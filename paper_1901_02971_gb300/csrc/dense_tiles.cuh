@@ -54,6 +54,9 @@ using TileSmem = TileSmemB<T, TB>;
 // UPPER: only the outputs on or above the diagonal of a diagonal tile are
 // needed (the patches whose row block lies entirely below their column
 // block are skipped and their accumulators stay zero).
+// FP64: row blocks at or beyond mi and the columns of warps at or beyond nj
+// are skipped too (uniform branches): the FP64 unit bounds these products, and
+// blocks of 7 to 60 rows would spend most of it on padding.
 template <typename T, bool UPPER = false, int B = TB>
 __device__ __forceinline__ void tn_acc(T (&acc)[4][TileGeom<B>::CB], const T* __restrict__ A, int lda, int mi,
                                        const T* __restrict__ Bm, int ldb, int nj, int K,
@@ -64,7 +67,7 @@ __device__ __forceinline__ void tn_acc(T (&acc)[4][TileGeom<B>::CB], const T* __
   constexpr int PR = G::PR, PC = G::PC, CB = G::CB, NTH = G::NTH;
   constexpr int NL = KC * B / NTH;  // elements of each operand loaded per thread per chunk
   const int tid = threadIdx.x;
-  const int tx = tid % PR, ty = tid / PR;
+  const int tx = tid % PR, ty = tid / PR, ty0 = (tid & ~31) / PR;  // ty0: first column of the warp's
   T ra[NL], rb[NL];
   auto load = [&](int k0) {
 #pragma unroll
@@ -100,7 +103,12 @@ __device__ __forceinline__ void tn_acc(T (&acc)[4][TileGeom<B>::CB], const T* __
       for (int ii = 0; ii < 4; ++ii)
 #pragma unroll
         for (int jj = 0; jj < CB; ++jj)
-          if (!UPPER || !G::below(ii, jj)) acc[ii][jj] = fma(av[ii], bv[jj], acc[ii][jj]);
+          if constexpr (sizeof(T) == 8) {
+            if ((!UPPER || !G::below(ii, jj)) && PR * ii < mi && ty0 + PC * jj < nj)
+              acc[ii][jj] = fma(av[ii], bv[jj], acc[ii][jj]);
+          } else {
+            if (!UPPER || !G::below(ii, jj)) acc[ii][jj] = fma(av[ii], bv[jj], acc[ii][jj]);
+          }
     }
     buf ^= 1;
   }
@@ -321,11 +329,12 @@ __device__ bool potrf_inv_tile(SqTileB<T, B>& s, SqTileB<T, B>& D, int nb) {
 // patch; starts and ends synchronised.  For l in the PR-row block lb, the
 // rows tx + PR ii with ii < lb lie above l, where D is zero, so their
 // products are skipped (uniformly over the CTA).
+// Only the rows < nb and the columns < nc matter (FP64 skips the others).
 template <typename T, int B>
-__device__ void apply_inv_tile(const SqTileB<T, B>& D, SqTileB<T, B>& Bt, int nb) {
+__device__ void apply_inv_tile(const SqTileB<T, B>& D, SqTileB<T, B>& Bt, int nb, int nc) {
   using G = TileGeom<B>;
   constexpr int PR = G::PR, PC = G::PC, CB = G::CB;
-  const int tx = threadIdx.x % PR, ty = threadIdx.x / PR;
+  const int tx = threadIdx.x % PR, ty = threadIdx.x / PR, ty0 = (threadIdx.x & ~31) / PR;
   T acc[4][CB];
   zero_acc(acc);
 #pragma unroll
@@ -340,7 +349,8 @@ __device__ void apply_inv_tile(const SqTileB<T, B>& D, SqTileB<T, B>& Bt, int nb
 #pragma unroll
       for (int ii = lb; ii < 4; ++ii)
 #pragma unroll
-        for (int jj = 0; jj < CB; ++jj) acc[ii][jj] = fma(dv[ii], bv[jj], acc[ii][jj]);
+        for (int jj = 0; jj < CB; ++jj)
+          if (sizeof(T) == 4 || (PR * ii < nb && ty0 + PC * jj < nc)) acc[ii][jj] = fma(dv[ii], bv[jj], acc[ii][jj]);
     }
   }
   __syncthreads();

@@ -27,6 +27,7 @@ struct RowDesc {      // a cluster's block row or its diagonal block
   int32_t bw2;        // the same in 32-tiles (FP64 pivot factorization)
   int32_t band;       // element half-bandwidth of the block (0 = dense or not known)
   int32_t pad;
+  const double* dinv32;  // k_inv_diag: the FP64 inverses U_kk^{-T} of the 32x32 diagonal tiles (nullptr: not at hand)
 };
 
 template <typename T>
@@ -135,7 +136,7 @@ __global__ void __launch_bounds__(TileGeom<B>::NTH) k_potrf_trsm(const RowDesc<T
   load_tile(D, d.dinv + (size_t)k * B * B, B, B, B);
   load_tile(Bt, d.R + k0 + (size_t)j0 * d.ld, d.ld, nb, nc);
   __syncthreads();
-  apply_inv_tile(D, Bt, nb);
+  apply_inv_tile(D, Bt, nb, nc);
   store_tile(Bt, d.R + k0 + (size_t)j0 * d.ld, d.ld, nb, nc);
   pdl_trigger();
 }
@@ -322,7 +323,10 @@ __global__ void __launch_bounds__(BAND_NT) k_potrf_band(const BandTask<TS>* __re
 // In 32 x 32 blocks, U^{-1} = [D11, -D11 U12 D22; 0, D22]: each diagonal
 // block is inverted by one warp, a lane per column by back substitution in
 // registers (no block barrier inside), then the corner by two 32 x 32
-// products, four 32 x 32 warps; the result is stored transposed.
+// products, four 32 x 32 warps; the result is stored transposed.  The tile
+// Cholesky leaves the inverses of its 32 x 32 diagonal tiles behind; where the
+// block was factored by it they take the place of the substitution, its longest
+// chain.  A tile of at most 32 rows has no corner to form.
 constexpr int INV_NT = 128;
 template <typename T>
 __global__ void __launch_bounds__(INV_NT) k_inv_diag(const RowDesc<T>* __restrict__ rows) {
@@ -339,7 +343,12 @@ __global__ void __launch_bounds__(INV_NT) k_inv_diag(const RowDesc<T>* __restric
     U.v[i][j] = (i < nb && j < nb) ? d.R[(k0 + i) + (size_t)(k0 + j) * d.ld] : (i == j ? T(1) : T(0));
   }
   __syncthreads();
-  if (warp < 2) {  // D_bb = U_bb^{-1}: column j = lane, rows i <= j
+  if (d.dinv32) {
+    for (int e = tid; e < 2 * 32 * 32; e += INV_NT) {
+      const int h = e >> 10, i = (e >> 5) & 31, j = e & 31, o = 32 * h;  // tile h, entry (j, i) of U_bb^{-T}
+      D.v[o + i][o + j] = o < nb ? (T)d.dinv32[((size_t)(2 * blockIdx.x + h) << 10) + (size_t)(32 * i + j)] : T(i == j);
+    }
+  } else if (warp < 2) {  // D_bb = U_bb^{-1}: column j = lane, rows i <= j
     const int o = 32 * warp, j = lane;
     const T rinv = T(1) / U.v[o + lane][o + lane];
     T x[32];
@@ -355,10 +364,16 @@ __global__ void __launch_bounds__(INV_NT) k_inv_diag(const RowDesc<T>* __restric
     for (int i = 0; i < 32; ++i) D.v[o + i][o + j] = x[i];
   }
   __syncthreads();
-  // W = U12 D22 into D's lower-left block (rows 32.., columns ..31)
+  // W = U12 D22 into D's lower-left block (rows 32.., columns ..31); zero when
+  // the tile has no rows there
   const int jc = lane, i0 = warp;  // thread: column jc, rows i0 + 4 m
+  if (nb <= 32) {
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
+    for (int m = 0; m < 8; ++m) D.v[i0 + 4 * m][32 + jc] = T(0);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int m = 0; m < 8 && nb > 32; ++m) {
     const int i = i0 + 4 * m;
     T acc = T(0);
     for (int k = 0; k <= jc; ++k) acc = fma(U.v[i][32 + k], D.v[32 + k][32 + jc], acc);
@@ -367,7 +382,7 @@ __global__ void __launch_bounds__(INV_NT) k_inv_diag(const RowDesc<T>* __restric
   __syncthreads();
   // D12 = -D11 W
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
+  for (int m = 0; m < 8 && nb > 32; ++m) {
     const int i = i0 + 4 * m;
     T acc = T(0);
     for (int k = i; k < 32; ++k) acc = fma(D.v[i][k], D.v[32 + k][jc], acc);
@@ -419,7 +434,7 @@ __global__ void __launch_bounds__(NT) k_trsm_cols(const TrsmTask<T>* __restrict_
         B.v[r][c] -= acc[ii][jj];
       }
     __syncthreads();
-    apply_inv_tile(U, B, nb);
+    apply_inv_tile(U, B, nb, nc);
     store_tile(B, X + i0, d.ldb, nb, nc);
     __syncthreads();
     const int i1 = i0 + TB;
@@ -483,52 +498,164 @@ __global__ void __launch_bounds__(NT) k_schur(const SchurTile* __restrict__ tile
   }
 }
 
+// The same update in two launches, each separator's couplings taken as one
+// block: G_s = X_s X_s^T over all its neighbours' columns at once (upper
+// triangle, 64 x 64 tiles; for TF32 operands k_schur_tma's tiles), then every
+// target block subtracts its pieces of the G's in the same fixed order.
+// A separator of a 3D grid has 26 and more neighbours of 1 to 64 dofs, one of a
+// graph over a hundred of a few dofs each: tiles per pair of neighbours are
+// mostly padding (64^3: 44 GFLOP executed for 25, of 29 with G; leaves of a
+// 50 000-point graph: 119 for 3.2, of 4.2), and the FP64 unit or, in FP32, the
+// latency of so many nearly empty tiles bound the update.  Schur family, tiles
+// per pair -> G: 64^3 FP64 37.6 -> 24.1 ms, TF32 1.36 -> 0.63, the graph (FP32)
+// 4.95 -> 0.52, 64 x 64 (FP64) 0.65 -> 0.21.
+template <typename T>
+struct GramTask {
+  const T* X;  // X^T: ns x m, leading dimension ld
+  T* G;        // m x m, leading dimension m; entries (i, j), i <= j, are set
+  int32_t ns, m, ld, pad;
+};
+template <typename T>
+__global__ void __launch_bounds__(NT) k_gram(const SchurTile* __restrict__ tiles, const GramTask<T>* __restrict__ tasks) {
+  __shared__ TileSmem<T> sm;
+  const SchurTile t = tiles[blockIdx.x];
+  const GramTask<T> d = tasks[t.block];
+  const int mi = min(TB, d.m - t.i0), nj = min(TB, d.m - t.j0);
+  T acc[4][4];
+  zero_acc(acc);
+  const T *A = d.X + (size_t)t.i0 * d.ld, *B = d.X + (size_t)t.j0 * d.ld;
+  if (t.i0 == t.j0) tn_acc<T, true>(acc, A, d.ld, mi, B, d.ld, nj, d.ns, sm);
+  else tn_acc(acc, A, d.ld, mi, B, d.ld, nj, d.ns, sm);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+  for (int jj = 0; jj < 4; ++jj)
+#pragma unroll
+    for (int ii = 0; ii < 4; ++ii) {
+      const int r = tx + 16 * ii, c = ty + 16 * jj;
+      if (r < mi && c < nj) d.G[(size_t)(t.i0 + r) + (size_t)(t.j0 + c) * d.m] = acc[ii][jj];
+    }
+}
+
+template <typename T>
+struct PullContrib {
+  const T* G;           // a separator's G
+  int32_t ldg, ia, ib;  // its size, first rows of a and of b
+  int32_t pad;
+};
+// One warp per 32 x 32 tile of a target block: C1 -= sum of its pieces, C2 = C1^T.
+constexpr int PULL_WARPS = 4;
+template <typename T>
+__global__ void __launch_bounds__(32 * PULL_WARPS) k_schur_pull(const SchurTile* __restrict__ tiles, int ntile,
+                                                                const SchurBlock<T>* __restrict__ blocks,
+                                                                const PullContrib<T>* __restrict__ contribs) {
+  __shared__ T s[PULL_WARPS][32][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = (int)blockIdx.x * PULL_WARPS + w;
+  if (g >= ntile) return;  // uniform over the warp; the warps never synchronise with each other
+  const SchurTile t = tiles[g];
+  const SchurBlock<T> b = blocks[t.block];
+  const int r = t.i0 + lane, nc = min(32, b.cols - t.j0);
+  const bool live = r < b.rows, diag = !b.C2;
+#pragma unroll 1
+  for (int c0 = 0; c0 < nc; c0 += 8) {
+    T acc[8], v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      acc[u] = T(0);
+      v[u] = live && c0 + u < nc ? b.C1[(size_t)r + (size_t)(t.j0 + c0 + u) * b.ld1] : T(0);
+    }
+    for (int e = b.cbeg; e < b.cend; ++e) {
+      const PullContrib<T> p = contribs[e];
+      const int i = p.ia + r, j = p.ib + t.j0 + c0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (!live || c0 + u >= nc) continue;
+        const bool sw = diag && i > j + u;  // below the diagonal of a == b: the mirrored entry
+        acc[u] += p.G[sw ? (size_t)(j + u) + (size_t)i * p.ldg : (size_t)i + (size_t)(j + u) * p.ldg];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (!live || c0 + u >= nc) continue;
+      const T x = v[u] - acc[u];
+      b.C1[(size_t)r + (size_t)(t.j0 + c0 + u) * b.ld1] = x;
+      s[w][c0 + u][lane] = x;
+    }
+  }
+  if (diag) return;
+  __syncwarp();
+  if (lane < nc)
+    for (int q = 0; q < min(32, b.rows - t.i0); ++q)
+      b.C2[(size_t)(t.j0 + lane) + (size_t)(t.i0 + q) * b.ld2] = s[w][lane][q];
+}
+
 // ---------------------------------------------------------------- two-sided scaling, second side
 
-// Scaling of an adjacent pair p < q (Sec. 2.5), second side: with
-// B = U_p^{-T} A_pq (|p| x |q|, the first side's block-row solve) and the
-// pivot inverse Y_q = U_q^{-T} (|q| x |q|, lower triangular, zero above the
-// diagonal in memory), the scaled block in q's row is
-// O = (U_p^{-T} A_pq U_q^{-1})^T = Y_q B^T (|q| x |p|).  One 64 x 64 tile of
-// O per CTA (tile list: task, i0, j0); K stops at the tile's last row, past
-// which Y_q is zero.
+// Scaling of the adjacent pairs p < q of one cluster q (Sec. 2.5), second
+// side: with B_p = U_p^{-T} A_pq (|p| x |q|, the first side's block-row solve)
+// and the pivot inverse Y_q = U_q^{-T} (|q| x |q|, lower triangular, zero above
+// the diagonal in memory), the scaled blocks in q's row are
+// O_p = (U_p^{-T} A_pq U_q^{-1})^T = Y_q B_p^T (|q| x |p|).  They are the first
+// columns of q's coupling, one after the other, so q is one product Y_q [B_p1^T
+// B_p2^T ...] of 64 x 64 tiles over those columns, each lane finding the row of
+// the p that its column belongs to (tiles per pair padded blocks of 7 to 60
+// columns to 64: 64^3, FP64 18.7 -> 13.2 ms, FP32 0.97 -> 0.70 ms).  K stops at the tile's last
+// row, past which Y_q is zero.  FP64 skips padding as tn_acc does.
+template <typename T>
+struct ScalePair {
+  const T* B;      // p's row at q's columns, leading dimension ldb
+  int32_t ldb, c;  // c: first column in q's product
+};
 template <typename T>
 struct ScaleTask {
-  const T* B;  // p's row at q's columns, leading dimension ldb
   const T* Y;  // Y_q, leading dimension ldy
-  T* O;        // q's row at p's columns, leading dimension ldo
-  int32_t ldb, ldo, np, nq, ldy, pad;
+  T* O;        // q's row at its first neighbour's columns, leading dimension ldo
+  int32_t ldo, nc, nq, ldy;  // nc: columns of all pairs
+  int32_t p0, p1;            // pairs [p0, p1)
 };
 
 template <typename T>
 __global__ void __launch_bounds__(NT) k_scale_gemm(const SchurTile* __restrict__ tiles,
-                                                   const ScaleTask<T>* __restrict__ tasks) {
+                                                   const ScaleTask<T>* __restrict__ tasks,
+                                                   const ScalePair<T>* __restrict__ pairs) {
   constexpr int KC2 = 16;
   __shared__ T ys[KC2][TB + 1], bs[KC2][TB + 1];
   const SchurTile tl = tiles[blockIdx.x];
   const ScaleTask<T> d = tasks[tl.block];
   const int i0 = tl.i0, j0 = tl.j0, tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
+  const int tx = tid & 15, ty = tid >> 4, ty0 = (tid & ~31) >> 4;
+  const int mi = min(TB, d.nq - i0), nj = min(TB, d.nc - j0);
   T acc[4][4];
   zero_acc(acc);
   const int kend = min(d.nq, i0 + TB);
   constexpr int NL = TB * KC2 / NT;  // elements of each operand per thread and chunk
+  const int li = tid & (TB - 1);     // this thread loads row li of Y's tile and column li of the product
+  const T* bp = nullptr;             // (0, k) of that column: bp[k ldb]
+  int ldb = 0;
+  if (li < nj) {
+    int lo = d.p0, hi = d.p1 - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (pairs[mid].c <= j0 + li) lo = mid; else hi = mid - 1;
+    }
+    const ScalePair<T> pr = pairs[lo];
+    bp = pr.B + (j0 + li - pr.c);
+    ldb = pr.ldb;
+  }
   T ry[NL], rb[NL];
-  auto load = [&](int k0) {  // Y(i0 + i, k0 + kk), B(j0 + i, k0 + kk): lanes along i
+  auto load = [&](int k0) {  // Y(i0 + li, k), B(j0 + li, k): lanes along the rows
 #pragma unroll
     for (int r = 0; r < NL; ++r) {
-      const int e = tid + NT * r, i = e & (TB - 1), k = k0 + e / TB;
-      ry[r] = (i0 + i < d.nq && k < kend) ? d.Y[(i0 + i) + (size_t)k * d.ldy] : T(0);
-      rb[r] = (j0 + i < d.np && k < kend) ? d.B[(j0 + i) + (size_t)k * d.ldb] : T(0);
+      const int k = k0 + tid / TB + NT / TB * r;
+      ry[r] = (li < mi && k < kend) ? d.Y[(i0 + li) + (size_t)k * d.ldy] : T(0);
+      rb[r] = (bp && k < kend) ? bp[(size_t)k * ldb] : T(0);
     }
   };
   if (kend > 0) load(0);
   for (int k0 = 0; k0 < kend; k0 += KC2) {
 #pragma unroll
     for (int r = 0; r < NL; ++r) {
-      const int e = tid + NT * r;
-      ys[e / TB][e & (TB - 1)] = ry[r];
-      bs[e / TB][e & (TB - 1)] = rb[r];
+      ys[tid / TB + NT / TB * r][li] = ry[r];
+      bs[tid / TB + NT / TB * r][li] = rb[r];
     }
     __syncthreads();
     if (k0 + KC2 < kend) load(k0 + KC2);  // the next chunk's loads overlap this chunk's products
@@ -543,16 +670,17 @@ __global__ void __launch_bounds__(NT) k_scale_gemm(const SchurTile* __restrict__
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
+        for (int b = 0; b < 4; ++b)
+          if (sizeof(T) == 4 || (16 * a < mi && ty0 + 16 * b < nj)) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int b = 0; b < 4; ++b)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int i = i0 + tx + 16 * a, j = j0 + ty + 16 * b;
-      if (i < d.nq && j < d.np) d.O[i + (size_t)j * d.ldo] = acc[a][b];
+    for (int a = 0; a < 4; ++a) {
+      const int i = tx + 16 * a, j = ty + 16 * b;
+      if (i < mi && j < nj) d.O[(i0 + i) + (size_t)(j0 + j) * d.ldo] = acc[a][b];
     }
 }
 

@@ -179,6 +179,10 @@ __global__ void __launch_bounds__(TC_NT, 4) k_schur_tma(const SchurTile* __restr
           const int col = c0 + j;
           if (col >= nj) break;
           const size_t o1 = (size_t)(t.i0 + row) + (size_t)(t.j0 + col) * b.ld1;
+          if (b.ld2 < 0) {  // G_s itself, for k_schur_pull
+            b.C1[o1] = __uint_as_float(r[j]);
+            continue;
+          }
           const float v = b.C1[o1] - __uint_as_float(r[j]);
           b.C1[o1] = v;
           T[row * (TC_N + 1) + col] = v;

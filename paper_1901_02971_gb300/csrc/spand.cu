@@ -67,6 +67,7 @@ constexpr size_t kCpqrChunkBudget = 224 * 1024;  // shared memory per sparsifica
 constexpr size_t kSmemPerSM = 228 * 1024;        // shared memory of one SM (each resident CTA also reserves 1 KB)
 constexpr int kCpqrMaxCluster = 8;              // thread-block cluster size (broadcasts to 16 CTAs cost 3.5x more)
 constexpr double kCqFp64Work = 2000;              // see its use
+constexpr size_t kGramBytes = size_t(4) << 30;    // most workspace for the separators' G blocks of a step
 constexpr int kAuxStreams = 8;
 constexpr double kCombineWork = 2e9;      // n^2 m of a step's separators up to which their G blocks are formed (FP32)
 constexpr double kApplyStreamBytes = 2e7;  // factor bytes of a phase of the apply from which it is LA_STREAM
@@ -797,7 +798,9 @@ static void pivot_chol(spand_handle h, const std::vector<RowDesc<T>>& rows, int*
       ++h->prof.launches;
     }
   }
-  inv_diag_batch<T>(h, rows, s);
+  std::vector<RowDesc<T>> inv(rows);
+  for (size_t i = 0; i < rows.size(); ++i) inv[i].dinv32 = r64[i].dinv;  // nullptr: factored by the banded kernel
+  inv_diag_batch<T>(h, inv, s);
 }
 
 template <typename T>
@@ -2256,10 +2259,48 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
                               lay.ld[sidx], TC_N))
             tma = false;
         }
+        // the separators' G (in the scratch buffer that step t + 1 will use),
+        // unless they would take more than kGramBytes, or BF16 operands
+        size_t gbytes = 0;
+        std::vector<size_t> goff(n, 0);
+        for (int sidx : seps) {
+          const size_t m = sz[sidx] > 0 ? (size_t)(lay.W[sidx] - sz[sidx]) : 0;
+          goff[sidx] = gbytes;
+          gbytes += align256(m * m * sizeof(T));
+        }
+        const bool gram = gbytes <= kGramBytes && (!tc || tma);
+        std::vector<GramTask<T>> gtask;
+        std::vector<SchurBlock<T>> gblock;  // TF32: G as the target of k_schur_tma
+        std::vector<PullContrib<T>> pulls;
+        std::vector<SchurTile> ptile;
+        char* gbase = gram ? (char*)h->scratch[(t + 1) & 1].ensure(gbytes) : nullptr;
         const int ti = tc ? TC_M : TB, tj = tc ? TC_N : TB;
-        for (size_t b = 0; b < blocks.size(); ++b) {
-          for (int i0 = 0; i0 < blocks[b].rows; i0 += ti)
-            for (int j0 = 0; j0 < blocks[b].cols; j0 += tj) tiles.push_back({(int32_t)b, i0, j0});
+        if (gram) {
+          for (int sidx : seps) {
+            const int m = sz[sidx] > 0 ? lay.W[sidx] - sz[sidx] : 0;
+            if (m <= 0) continue;
+            T* G = (T*)(gbase + goff[sidx]);
+            const int32_t id = (int32_t)gtask.size();
+            gtask.push_back({lay.row[sidx] + (size_t)sz[sidx] * lay.ld[sidx], G, sz[sidx], m, lay.ld[sidx], 0});
+            if (tc) gblock.push_back({G, nullptr, m, -1, m, m, id, id + 1});
+            for (int i0 = 0; i0 < m; i0 += ti)
+              for (int j0 = i0 / tj * tj; j0 < m; j0 += tj) tiles.push_back({id, i0, j0});
+          }
+          pulls.reserve(flat.size());
+          for (const SchurContrib<T>& c : flat) {
+            const int sidx = c.owner;
+            const T* X0 = lay.row[sidx] + (size_t)sz[sidx] * lay.ld[sidx];
+            pulls.push_back({(const T*)(gbase + goff[sidx]), lay.W[sidx] - sz[sidx], (int32_t)((c.Xa - X0) / c.lds),
+                             (int32_t)((c.Xb - X0) / c.lds), 0});
+          }
+          for (size_t b = 0; b < blocks.size(); ++b)
+            for (int i0 = 0; i0 < blocks[b].rows; i0 += 32)
+              for (int j0 = 0; j0 < blocks[b].cols; j0 += 32) ptile.push_back({(int32_t)b, i0, j0});
+        } else {
+          for (size_t b = 0; b < blocks.size(); ++b) {
+            for (int i0 = 0; i0 < blocks[b].rows; i0 += ti)
+              for (int j0 = 0; j0 < blocks[b].cols; j0 += tj) tiles.push_back({(int32_t)b, i0, j0});
+          }
         }
         const CUtensorMap* dmaps = nullptr;
         if (tma) {
@@ -2268,7 +2309,17 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           dmaps = at<const CUtensorMap>(upload<T>(h, pkm, s), om);
         }
         std::vector<SchurContribTma> flat_tma;
-        if (tma) {
+        if (tma && gram) {
+          for (int sidx : seps) {
+            if (sz[sidx] <= 0 || lay.W[sidx] <= sz[sidx]) continue;
+            SchurContribTma m{};
+            m.map_a = dmaps + tmap_of[sidx];
+            m.map_b = dmaps + tmap_of[sidx] + 1;
+            m.col_a = m.col_b = sz[sidx];
+            m.ns = sz[sidx];
+            flat_tma.push_back(m);
+          }
+        } else if (tma) {
           flat_tma.reserve(flat.size());
           for (const SchurContrib<T>& c : flat) {
             // the separator row is the one whose columns Xa, Xb point into
@@ -2283,7 +2334,8 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           }
         }
         Packer pk;
-        size_t ob = pk.add(blocks), oc = tma ? pk.add(flat_tma) : pk.add(flat), ot = pk.add(tiles);
+        size_t ob = pk.add(blocks), oc = tma ? pk.add(flat_tma) : gram ? pk.add(gtask) : pk.add(flat), ot = pk.add(tiles);
+        const size_t og = pk.add(gblock), op = pk.add(pulls), opt = pk.add(ptile);
         void* d = upload<T>(h, pk, s);
         double fl = 0, by = 0;
         for (auto& bl : blocks) {
@@ -2298,7 +2350,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
             const void* fn = (const void*)k_schur_tma;
             ensure_smem(fn, TM_SMEM);
             const SchurTile* a0 = at<const SchurTile>(d, ot);
-            const SchurBlock<float>* a1 = at<const SchurBlock<float>>(d, ob);
+            const SchurBlock<float>* a1 = at<const SchurBlock<float>>(d, gram ? og : ob);
             const SchurContribTma* a2 = at<const SchurContribTma>(d, oc);
             int* a3 = d_info;  // [0]: a bounded wait gave up
             void* args[] = {(void*)&a0, (void*)&a1, (void*)&a2, (void*)&a3};
@@ -2315,12 +2367,20 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
             CK(cudaLaunchKernel(fn, dim3((unsigned)tiles.size()), dim3(TC_NT), args, tsm, s));
           }
         }
-        if (!tc)
+        if (!tc && gram)
+          k_gram<T><<<(unsigned)tiles.size(), NT, 0, s>>>(at<const SchurTile>(d, ot), at<const GramTask<T>>(d, oc));
+        else if (!tc)
           k_schur<T><<<(unsigned)tiles.size(), NT, 0, s>>>(at<const SchurTile>(d, ot), at<const SchurBlock<T>>(d, ob),
                                                           at<const SchurContrib<T>>(d, oc));
         CKLAUNCH();
-        h->prof.launches += 1;
-        h->prof.end(pid, s, fl, by, 1);
+        if (gram) {
+          const int np = (int)ptile.size();
+          k_schur_pull<T><<<(unsigned)((np + PULL_WARPS - 1) / PULL_WARPS), 32 * PULL_WARPS, 0, s>>>(
+              at<const SchurTile>(d, opt), np, at<const SchurBlock<T>>(d, ob), at<const PullContrib<T>>(d, op));
+          CKLAUNCH();
+        }
+        h->prof.launches += gram ? 2 : 1;
+        h->prof.end(pid, s, fl, by, gram ? 2 : 1);
       }
     }
     CK(cudaEventRecord(tm.at(t, 1), s));
@@ -2424,7 +2484,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       std::vector<RowDesc<T>> diag, ident;
       std::vector<int> diag_cl;
       std::vector<TrsmTask<T>> up;
-      std::vector<CopyTask<T>> m_up, m_lo;  // per pair p < q: p -> q (the product's operands), q -> p
+      std::vector<CopyTask<T>> m_lo;  // per pair p < q: the scaled block from q's row into p's, transposed
       std::vector<RowDesc<T>> idr;
       for (int p : rems) {
         if (sz[p] <= 0 || h->opts.variant == SPAND_IN) continue;  // In: no block scaling
@@ -2437,23 +2497,14 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           const int32_t q = lay.nidx[e];
           if (q <= p || sz[q] <= 0) continue;
           const int32_t oqp = lay.off_of(q, p);
-          CopyTask<T> c;
-          c.src = lay.row[p] + (size_t)lay.noff[e] * lay.ld[p];
-          c.dst = lay.row[q] + (size_t)oqp * lay.ld[q];
-          c.lds = lay.ld[p];
-          c.ldd = lay.ld[q];
-          c.rows = sz[q];
-          c.cols = sz[p];
-          c.trans = 1;
-          c.pad = 0;
-          m_up.push_back(c);
-          CopyTask<T> b = c;
-          b.src = c.dst;
-          b.dst = const_cast<T*>(c.src);
+          CopyTask<T> b{};
+          b.src = lay.row[q] + (size_t)oqp * lay.ld[q];
+          b.dst = lay.row[p] + (size_t)lay.noff[e] * lay.ld[p];
           b.lds = lay.ld[q];
           b.ldd = lay.ld[p];
           b.rows = sz[p];
           b.cols = sz[q];
+          b.trans = 1;
           m_lo.push_back(b);
         }
         const int ldy = row_ld(sz[p]);
@@ -2473,36 +2524,32 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         stt.mem_f += (int64_t)sz[p] * (sz[p] + 1) / 2;
       }
       // second side of every pair p < q from the first side's block and Y_q:
-      // O = Y_q (U_p^{-T} A_pq)^T into q's row (the scaled A_qp)
+      // O = Y_q (U_p^{-T} A_pq)^T into q's row (the scaled A_qp), all pairs of
+      // q as one product
       std::vector<ScaleTask<T>> sct;
+      std::vector<ScalePair<T>> scp;
       std::vector<SchurTile> sctl;
-      {
-        std::vector<const T*> yof(n, nullptr);
-        for (size_t i = 0; i < sq_cluster.size(); ++i) yof[sq_cluster[i]] = sqops[i].Y;
-        for (const CopyTask<T>& c : m_up) {  // one per pair p < q: src = p's block, dst = q's block
-          ScaleTask<T> k;
-          k.B = c.src;
-          k.O = c.dst;
-          k.ldb = c.lds;
-          k.ldo = c.ldd;
-          k.np = c.cols;
-          k.nq = c.rows;
-          k.Y = nullptr;
-          k.ldy = row_ld(c.rows);
-          sct.push_back(k);
+      for (int q : rems) {
+        if (!ypin[q]) continue;
+        ScaleTask<T> k{};
+        k.p0 = (int32_t)scp.size();
+        for (int32_t e = lay.nptr[q]; e < lay.nptr[q + 1]; ++e) {
+          const int32_t p = lay.nidx[e];
+          if (p >= q) break;
+          if (sz[p] <= 0) continue;
+          if (!k.O) k.O = lay.row[q] + (size_t)lay.noff[e] * lay.ld[q];
+          scp.push_back({lay.row[p] + (size_t)lay.off_of(p, q) * lay.ld[p], lay.ld[p], k.nc});
+          k.nc += sz[p];
         }
-        size_t i = 0;
-        for (int p : rems) {
-          if (sz[p] <= 0 || h->opts.variant == SPAND_IN) continue;
-          for (int32_t e = lay.nptr[p]; e < lay.nptr[p + 1]; ++e) {
-            const int32_t q = lay.nidx[e];
-            if (q <= p || sz[q] <= 0) continue;
-            sct[i++].Y = yof[q];
-          }
-        }
-        for (size_t k = 0; k < sct.size(); ++k)
-          for (int i0 = 0; i0 < sct[k].nq; i0 += TB)
-            for (int j0 = 0; j0 < sct[k].np; j0 += TB) sctl.push_back({(int32_t)k, i0, j0});
+        k.p1 = (int32_t)scp.size();
+        if (k.nc == 0) continue;
+        k.Y = ypin[q];
+        k.ldo = lay.ld[q];
+        k.nq = sz[q];
+        k.ldy = row_ld(sz[q]);
+        for (int i0 = 0; i0 < k.nq; i0 += TB)
+          for (int j0 = 0; j0 < k.nc; j0 += TB) sctl.push_back({(int32_t)sct.size(), i0, j0});
+        sct.push_back(k);
       }
       set_identity<T>(h, ident, s);
       pivot_chol<T>(h, diag, d_info + 2 * t + 1, s);
@@ -2510,13 +2557,14 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       trsm_batch<T>(h, up, s);   // upper blocks U_p^{-T} A_pq and the inverses Y_p
       if (!sctl.empty()) {
         Packer pks;
-        const size_t okt = pks.add(sct), okl = pks.add(sctl);
+        const size_t okt = pks.add(sct), okl = pks.add(sctl), okp = pks.add(scp);
         void* dks = upload<T>(h, pks, s);
         double fl = 0;
-        for (const ScaleTask<T>& k : sct) fl += (double)k.nq * k.nq * k.np;
+        for (const ScaleTask<T>& k : sct) fl += (double)k.nq * k.nq * k.nc;
         const int pid = h->prof.begin(F_TRSM, s);
         k_scale_gemm<T><<<(unsigned)sctl.size(), NT, 0, s>>>(at<const SchurTile>(dks, okl),
-                                                             at<const ScaleTask<T>>(dks, okt));
+                                                             at<const ScaleTask<T>>(dks, okt),
+                                                             at<const ScalePair<T>>(dks, okp));
         CKLAUNCH();
         h->prof.launches += 1;
         h->prof.end(pid, s, fl, 0.0, 1);

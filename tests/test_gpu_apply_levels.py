@@ -41,3 +41,24 @@ def test_exact_apply_is_the_inverse(cuda_ok, dim, n, levels, precision):
     u = 2.0 ** (-53 if precision == "fp64" else -24)
     err = np.linalg.norm(z - ref) / np.linalg.norm(ref)
     assert err <= 20 * _cond(dim, n) * u, err
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "tf32"])
+@pytest.mark.parametrize("dim,n,levels,skip", [(2, 33, 6, 5), (3, 13, 5, 2), (3, 17, 4, 3), (2, 65, 4, 0)])
+def test_unscaled_steps_and_wide_couplings(cuda_ok, dim, n, levels, skip, precision):
+    """skip > 0: the clusters of the first steps pass through the apply unscaled,
+    next to scaled ones; couplings of one to several 64-column tiles with ragged
+    ends through the elimination's G blocks, the pull and the scaling product.
+    TF32 operands of the Schur update carry 2^-11."""
+    import torch
+    p = I.laplacian_2d(n) if dim == 2 else I.laplacian_3d(n)
+    r = I.rhs(p.n, 4)
+    ref = sla.spsolve(p.to_scipy().tocsc(), r)
+    s = Solver.from_problem(p, levels=levels, eps=0.0, skip=skip, precision=precision).factorize()
+    try:
+        z = s.apply(torch.from_numpy(r).cuda()).cpu().numpy()
+    finally:
+        s.close()
+    u = 2.0 ** {"fp64": -53, "fp32": -24, "tf32": -11}[precision]
+    err = np.linalg.norm(z - ref) / np.linalg.norm(ref)
+    assert err <= 20 * _cond(dim, n) * u, err
