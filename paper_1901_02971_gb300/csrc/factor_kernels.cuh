@@ -684,6 +684,36 @@ __global__ void __launch_bounds__(NT) k_scale_gemm(const SchurTile* __restrict__
     }
 }
 
+// The scaled blocks of q's row back into the rows of the p's, transposed, over
+// the same tiles (the product reads p's blocks, so it cannot write them itself).
+template <typename T>
+__global__ void __launch_bounds__(NT) k_scale_mirror(const SchurTile* __restrict__ tiles,
+                                                     const ScaleTask<T>* __restrict__ tasks,
+                                                     const ScalePair<T>* __restrict__ pairs) {
+  __shared__ T s[TB][TB + 1];
+  const SchurTile tl = tiles[blockIdx.x];
+  const ScaleTask<T> d = tasks[tl.block];
+  const int i0 = tl.i0, j0 = tl.j0, tid = threadIdx.x, li = tid & (TB - 1);
+  const int mi = min(TB, d.nq - i0), nj = min(TB, d.nc - j0);
+  for (int j = tid / TB; j < nj; j += NT / TB)
+    if (li < mi) s[j][li] = d.O[(i0 + li) + (size_t)(j0 + j) * d.ldo];
+  T* bp = nullptr;
+  int ldb = 0;
+  if (li < nj) {
+    int lo = d.p0, hi = d.p1 - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (pairs[mid].c <= j0 + li) lo = mid; else hi = mid - 1;
+    }
+    const ScalePair<T> pr = pairs[lo];
+    bp = const_cast<T*>(pr.B) + (j0 + li - pr.c);
+    ldb = pr.ldb;
+  }
+  __syncthreads();
+  if (bp)
+    for (int i = tid / TB; i < mi; i += NT / TB) bp[(size_t)(i0 + i) * ldb] = s[li][i];
+}
+
 // ---------------------------------------------------------------- copies
 
 // Block copies in 32 x 32 tiles, one warp per tile: tile g = CP_WARPS

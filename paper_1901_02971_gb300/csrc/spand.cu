@@ -435,6 +435,27 @@ struct VecPool {
   }
 };
 
+// A factorization's larger descriptor arrays, kept from step to step and call
+// to call: they run to megabytes where the cluster graph is dense, and fresh
+// allocations of that size pay first-touch page faults each time.
+template <typename T>
+struct HostScratch {
+  std::vector<TrsmTask<T>> elim_trsm, scale_trsm;
+  std::vector<SchurBlock<T>> blocks;
+  std::vector<SchurContrib<T>> flat;
+  std::vector<PullContrib<T>> pulls;
+  std::vector<SchurTile> tiles, ptile, sctl;
+  std::vector<ScaleTask<T>> sct;
+  std::vector<ScalePair<T>> scp;
+  std::vector<CpqrNbr<T>> nbrs;
+  std::vector<CopyTask<T>> cps;
+  template <typename X>
+  static std::vector<X>& fresh(std::vector<X>& v) {
+    v.clear();
+    return v;
+  }
+};
+
 struct spand_handle_s {
   spand_opts opts{};
   int64_t n = 0, nnz = 0;
@@ -486,6 +507,16 @@ struct spand_handle_s {
     std::vector<int32_t> ptr, b, src, tgt;  // per entry of rems: ptr[i] .. ptr[i + 1]
   };
   std::vector<MergePlan> mplan;
+  // Per step, for every edge (p, q) of the layout between remaining clusters
+  // the index of (q, p) (-1 otherwise); fixed by the analysis.
+  std::vector<std::vector<int32_t>> rplan;
+  HostScratch<float> hs32;
+  HostScratch<double> hs64;
+  template <typename T>
+  HostScratch<T>& hs() {
+    if constexpr (std::is_same<T, double>::value) return hs64;
+    else return hs32;
+  }
   VecPool<int64_t> pool64;
   VecPool<std::pair<int32_t, int64_t>> poolpair;
   VecPool<ApplyItem> poolitem;
@@ -2038,6 +2069,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
   stt.factor_flops = 0;
   stt.fail_step = 0;
   stt.fail_cluster = -1;
+  HostScratch<T>& hs = h->template hs<T>();
   StepTimer tm(L);
   h->stage.reset();  // the previous factorization ended with a stream synchronisation
   // non-positive pivot flags per step: [2t] elimination pivots, [2t+1]
@@ -2132,7 +2164,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       std::vector<RowDesc<T>> diag, ident;
       std::vector<int> diag_cl;
       std::vector<double> diag_fl, tr_fl;
-      std::vector<TrsmTask<T>> tr_tasks;
+      std::vector<TrsmTask<T>>& tr_tasks = hs.fresh(hs.elim_trsm);
       for (int sidx : seps) {
         if (sz[sidx] <= 0) continue;
         const double ns = sz[sidx], m = lay.W[sidx] - sz[sidx];
@@ -2203,10 +2235,8 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         }
         plan.built = true;
       }
-      std::vector<SchurBlock<T>> blocks;
-      std::vector<SchurContrib<T>> flat;
-      blocks.reserve(plan.a.size());
-      flat.reserve(plan.csep.size());
+      std::vector<SchurBlock<T>>& blocks = hs.fresh(hs.blocks);
+      std::vector<SchurContrib<T>>& flat = hs.fresh(hs.flat);
       for (size_t id = 0; id < plan.a.size(); ++id) {
         const int32_t a = plan.a[id], b = plan.b[id];
         if (sz[a] <= 0 || sz[b] <= 0) continue;
@@ -2235,7 +2265,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         blocks.push_back(bl);
       }
       if (!blocks.empty()) {
-        std::vector<SchurTile> tiles;
+        std::vector<SchurTile>& tiles = hs.fresh(hs.tiles);
         // tensor cores for the TF32 / BF16 forms: 128 x 64 tiles; FP32 and
         // FP64 on the SIMT pipes: 64 x 64 tiles
         bool tc = sizeof(T) == 4 && (h->opts.precision == SPAND_TF32 || h->opts.precision == SPAND_BF16);
@@ -2271,8 +2301,8 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         const bool gram = gbytes <= kGramBytes && (!tc || tma);
         std::vector<GramTask<T>> gtask;
         std::vector<SchurBlock<T>> gblock;  // TF32: G as the target of k_schur_tma
-        std::vector<PullContrib<T>> pulls;
-        std::vector<SchurTile> ptile;
+        std::vector<PullContrib<T>>& pulls = hs.fresh(hs.pulls);
+        std::vector<SchurTile>& ptile = hs.fresh(hs.ptile);
         char* gbase = gram ? (char*)h->scratch[(t + 1) & 1].ensure(gbytes) : nullptr;
         const int ti = tc ? TC_M : TB, tj = tc ? TC_N : TB;
         if (gram) {
@@ -2286,7 +2316,6 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
             for (int i0 = 0; i0 < m; i0 += ti)
               for (int j0 = i0 / tj * tj; j0 < m; j0 += tj) tiles.push_back({id, i0, j0});
           }
-          pulls.reserve(flat.size());
           for (const SchurContrib<T>& c : flat) {
             const int sidx = c.owner;
             const T* X0 = lay.row[sidx] + (size_t)sz[sidx] * lay.ld[sidx];
@@ -2481,10 +2510,16 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
     std::vector<T*> ypin(n, nullptr);       // per scaled cluster: its pivot inverse
     std::vector<T*> pfac(n, nullptr);       // per cluster: P_p in the factor (nullptr: not sparsified)
     if (sparsify) {
+      if (h->rplan.size() < (size_t)L + 1) h->rplan.resize((size_t)L + 1);
+      std::vector<int32_t>& rev = h->rplan[t];
+      if (rev.empty()) {
+        rev.assign(lay.nidx.size() + 1, -1);
+        for (int p : rems)
+          for (int32_t e = lay.nptr[p]; e < lay.nptr[p + 1]; ++e) rev[e] = lay.edge_of(lay.nidx[e], p);
+      }
       std::vector<RowDesc<T>> diag, ident;
       std::vector<int> diag_cl;
-      std::vector<TrsmTask<T>> up;
-      std::vector<CopyTask<T>> m_lo;  // per pair p < q: the scaled block from q's row into p's, transposed
+      std::vector<TrsmTask<T>>& up = hs.fresh(hs.scale_trsm);
       std::vector<RowDesc<T>> idr;
       for (int p : rems) {
         if (sz[p] <= 0 || h->opts.variant == SPAND_IN) continue;  // In: no block scaling
@@ -2493,20 +2528,6 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         diag_cl.push_back(p);
         const int fu = lay.first_upper(p);
         add_panels(up, lay.row[p], (const T*)dv, sz[p], lay.ld[p], fu, lay.W[p]);
-        for (int32_t e = lay.nptr[p]; e < lay.nptr[p + 1]; ++e) {
-          const int32_t q = lay.nidx[e];
-          if (q <= p || sz[q] <= 0) continue;
-          const int32_t oqp = lay.off_of(q, p);
-          CopyTask<T> b{};
-          b.src = lay.row[q] + (size_t)oqp * lay.ld[q];
-          b.dst = lay.row[p] + (size_t)lay.noff[e] * lay.ld[p];
-          b.lds = lay.ld[q];
-          b.ldd = lay.ld[p];
-          b.rows = sz[p];
-          b.cols = sz[q];
-          b.trans = 1;
-          m_lo.push_back(b);
-        }
         const int ldy = row_ld(sz[p]);
         T* Y = (T*)h->persist.alloc((size_t)ldy * sz[p] * sizeof(T));
         ident.push_back({Y, sz[p], ldy, nullptr});
@@ -2526,9 +2547,9 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       // second side of every pair p < q from the first side's block and Y_q:
       // O = Y_q (U_p^{-T} A_pq)^T into q's row (the scaled A_qp), all pairs of
       // q as one product
-      std::vector<ScaleTask<T>> sct;
-      std::vector<ScalePair<T>> scp;
-      std::vector<SchurTile> sctl;
+      std::vector<ScaleTask<T>>& sct = hs.fresh(hs.sct);
+      std::vector<ScalePair<T>>& scp = hs.fresh(hs.scp);
+      std::vector<SchurTile>& sctl = hs.fresh(hs.sctl);
       for (int q : rems) {
         if (!ypin[q]) continue;
         ScaleTask<T> k{};
@@ -2538,7 +2559,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           if (p >= q) break;
           if (sz[p] <= 0) continue;
           if (!k.O) k.O = lay.row[q] + (size_t)lay.noff[e] * lay.ld[q];
-          scp.push_back({lay.row[p] + (size_t)lay.off_of(p, q) * lay.ld[p], lay.ld[p], k.nc});
+          scp.push_back({lay.row[p] + (size_t)lay.noff[rev[e]] * lay.ld[p], lay.ld[p], k.nc});
           k.nc += sz[p];
         }
         k.p1 = (int32_t)scp.size();
@@ -2566,10 +2587,13 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
                                                              at<const ScaleTask<T>>(dks, okt),
                                                              at<const ScalePair<T>>(dks, okp));
         CKLAUNCH();
-        h->prof.launches += 1;
-        h->prof.end(pid, s, fl, 0.0, 1);
+        k_scale_mirror<T><<<(unsigned)sctl.size(), NT, 0, s>>>(at<const SchurTile>(dks, okl),
+                                                               at<const ScaleTask<T>>(dks, okt),
+                                                               at<const ScalePair<T>>(dks, okp));
+        CKLAUNCH();
+        h->prof.launches += 2;
+        h->prof.end(pid, s, fl, 0.0, 2);
       }
-      copy_batch<T>(h, m_lo, s);
       set_identity<T>(h, idr, s);
       CK(cudaEventRecord(tm.at(t, 2), s));
       // ---- sparsify, colour by colour (Sec. 2.6.1)
@@ -2591,7 +2615,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       }
       auto colour_of = [&](int p) { return sim ? 0 : (int)st.colour[p]; };
       std::vector<CpqrTask<T>> tasks;
-      std::vector<CpqrNbr<T>> nbrs;
+      std::vector<CpqrNbr<T>>& nbrs = hs.fresh(hs.nbrs);
       std::vector<int> tclass;  // cluster size of each task
       std::vector<int> tres;    // 1: the task's chunk lives in shared memory
       std::vector<int> treg;    // lane-group size of the register-resident kernel (0: chunked kernel)
@@ -2617,7 +2641,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           nb.Rq = lay.row[q];
           nb.q = q;
           nb.off_pq = lay.noff[e];
-          nb.off_qp = lay.off_of(q, p);
+          nb.off_qp = rev[e] < 0 ? -1 : lay.noff[rev[e]];
           if (nb.off_qp < 0) throw Fail{SPAND_ERR_STATE, "asymmetric block pattern"};
           nb.ldq = lay.ld[q];
           nbrs.push_back(nb);
@@ -3089,8 +3113,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         }
         mp.built = true;
       }
-      std::vector<CopyTask<T>> cps;
-      cps.reserve(mp.b.size());
+      std::vector<CopyTask<T>>& cps = hs.fresh(hs.cps);
       for (size_t ia = 0; ia < rems.size(); ++ia) {
         const int a = rems[ia];
         if (sz_after[a] <= 0) continue;
