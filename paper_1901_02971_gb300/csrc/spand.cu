@@ -533,7 +533,7 @@ struct spand_handle_s {
   cudaStream_t aux[kAuxStreams] = {};
   cudaEvent_t ev_fork = nullptr, ev_join[kAuxStreams] = {};
   cudaStream_t qs = nullptr;                         // Q_pc formation, one colour behind the QR kernels
-  cudaEvent_t ev_q = nullptr, ev_qdone = nullptr;
+  cudaEvent_t ev_q = nullptr;
   KProf prof;
   // the preconditioner apply program (phases of every step, on the device);
   // one cooperative launch of k_apply runs it
@@ -549,8 +549,8 @@ struct spand_handle_s {
   int apply_ctas = 0;        // CTAs per SM of the apply: 0 = not chosen yet (autotuned at the first apply)
   size_t apply_smem = 0;
   DevBuf d_bar;  // [0] grid-barrier arrival counter, [2] barrier-timeout flag
-  DevBuf d_qc;   // Q_pc of a step's interfaces (written and read on the side stream qs)
-  cudaEvent_t ev_comb = nullptr;  // the last k_combine launch
+  DevBuf d_qc;   // the reflectors (V, tau) and Q_pc of a step's interfaces, read on the side stream qs
+  cudaEvent_t ev_comb = nullptr;  // the last k_form_q or k_combine launch
   unsigned apply_spin_limit = kBarrierSpins;  // polls per grid-barrier wait of the apply
   unsigned apply_bias = 0;                    // 1: failure-path test, no barrier completes
   ~spand_handle_s() {
@@ -558,7 +558,6 @@ struct spand_handle_s {
       if (a) cudaStreamDestroy(a);
     if (qs) cudaStreamDestroy(qs);
     if (ev_q) cudaEventDestroy(ev_q);
-    if (ev_qdone) cudaEventDestroy(ev_qdone);
     if (ev_comb) cudaEventDestroy(ev_comb);
     if (ev_fork) cudaEventDestroy(ev_fork);
     for (auto& e : ev_join)
@@ -645,7 +644,6 @@ static void ensure_streams(spand_handle h) {
   for (auto& a : h->aux) CK(cudaStreamCreateWithFlags(&a, cudaStreamNonBlocking));
   CK(cudaStreamCreateWithFlags(&h->qs, cudaStreamNonBlocking));
   CK(cudaEventCreateWithFlags(&h->ev_q, cudaEventDisableTiming));
-  CK(cudaEventCreateWithFlags(&h->ev_qdone, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&h->ev_comb, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
   for (auto& e : h->ev_join) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -2057,6 +2055,8 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
   const int L = tr.L;
   const double eps = h->opts.eps;
   const int skip = h->opts.skip;
+  // a failed factorization may have left work on the side stream
+  if (h->ev_comb) CK(cudaStreamWaitEvent(s, h->ev_comb, 0));
   h->persist.reset();
   h->descs.reset();
   std::vector<ApplyStep<T>> apply;
@@ -2670,8 +2670,8 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         const bool resident = res_smem(C) <= CB;
         WOff w;
         w.nrm = 0;
-        w.v = wbytes; wbytes += align256((size_t)sz[p] * sz[p] * sizeof(T));
-        w.tau = wbytes; wbytes += align256((size_t)sz[p] * sizeof(T));
+        w.v = qbytes; qbytes += align256((size_t)sz[p] * sz[p] * sizeof(T));
+        w.tau = qbytes; qbytes += align256((size_t)sz[p] * sizeof(T));
         w.qc = qbytes; qbytes += align256((size_t)sz[p] * sz[p] * sizeof(T));
         w.gw = wbytes;
         if (!resident && !interp) wbytes += align256((size_t)C * Lp * ((mm + C - 1) / C) * sizeof(T));
@@ -2784,10 +2784,10 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       if (!tasks.empty()) {
         char* wb = interp ? nullptr : (char*)h->scratch[(t + 1) & 1].ensure(wbytes);
         char* qb = interp ? nullptr : (char*)h->d_qc.ensure(qbytes);
-        if (h->ev_comb) CK(cudaStreamWaitEvent(s, h->ev_comb, 0));  // the previous step's Q_pc have been read
+        if (h->ev_comb) CK(cudaStreamWaitEvent(s, h->ev_comb, 0));  // the previous step's reflectors and Q_pc have been read
         for (size_t i = 0; i < tasks.size() && wb; ++i) {
-          tasks[i].V = (T*)(wb + woff[i].v);
-          tasks[i].tau = (T*)(wb + woff[i].tau);
+          tasks[i].V = (T*)(qb + woff[i].v);
+          tasks[i].tau = (T*)(qb + woff[i].tau);
           tasks[i].Qc = (T*)(qb + woff[i].qc);
           tasks[i].gwork = (T*)(wb + woff[i].gw);
           cp_qc.push_back(tasks[i].Qc);
@@ -2851,14 +2851,17 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         ensure_streams(h);
         cpqr_pid = h->prof.begin(F_CPQR, s);
         size_t gi = 0;
-        int64_t nformq = 0;  // k_form_q launches (one per colour)
+        int64_t nformq = 0;  // k_form_q launches
+        size_t qbeg = 0;     // interfaces list[qbeg ..) still want their Q_pc
         while (gi < groups.size()) {  // one colour at a time; its groups run side by side
           size_t ge = gi;
           while (ge < groups.size() && groups[ge].colour == groups[gi].colour) ++ge;
-          CK(cudaEventRecord(h->ev_fork, s));
+          // the colour's first group stays on s (most colours have only one:
+          // no event, no hop between streams on the chain of colours)
+          if (ge > gi + 1) CK(cudaEventRecord(h->ev_fork, s));
           for (size_t g = gi; g < ge; ++g) {
-            cudaStream_t as = h->aux[(g - gi) % kAuxStreams];
-            CK(cudaStreamWaitEvent(as, h->ev_fork, 0));
+            cudaStream_t as = g == gi ? s : h->aux[(g - gi - 1) % kAuxStreams];
+            if (g != gi) CK(cudaStreamWaitEvent(as, h->ev_fork, 0));
             const Group& G = groups[g];
             const size_t smem = G.smem;
             // 512 threads for one- and two-CTA interfaces (latency hiding)
@@ -2903,16 +2906,17 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
             T a4 = (T)eps;
             void* args[] = {(void*)&a0, (void*)&a1, (void*)&a2, (void*)&d_cur, (void*)&a4};
             CK(cudaLaunchKernelExC(&cfg, fn, args));
-            CK(cudaEventRecord(h->ev_join[(g - gi) % kAuxStreams], as));
+            if (g != gi) CK(cudaEventRecord(h->ev_join[(g - gi - 1) % kAuxStreams], as));
           }
-          for (size_t g = gi; g < std::min(ge, gi + (size_t)kAuxStreams); ++g)
-            CK(cudaStreamWaitEvent(s, h->ev_join[(g - gi) % kAuxStreams], 0));
-          // Q_pc of this colour's interfaces on the side stream, overlapping
-          // the next colour's QR (nothing in the factorization reads Q_pc
-          // before the compaction below)
-          {
+          for (size_t g = gi + 1; g < std::min(ge, gi + 1 + (size_t)kAuxStreams); ++g)
+            CK(cudaStreamWaitEvent(s, h->ev_join[(g - gi - 1) % kAuxStreams], 0));
+          // Q_pc on the side stream, overlapping the next colours' QR (nothing
+          // on s reads it), for enough interfaces at a time to be worth a launch
+          const size_t qdone = ge < groups.size() ? gbeg[ge] : list.size();
+          if (qdone - qbeg >= (size_t)num_sms() || ge == groups.size()) {
             constexpr int NTQ = 256, NWQ = NTQ / 32;
-            const size_t l0 = gbeg[gi], l1 = ge < groups.size() ? gbeg[ge] : list.size();
+            const size_t l0 = qbeg, l1 = qdone;
+            qbeg = qdone;
             int kmx = 0;
             size_t need = 0;
             for (size_t li = l0; li < l1; ++li) {
@@ -2936,8 +2940,8 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           }
           gi = ge;
         }
-        CK(cudaEventRecord(h->ev_qdone, h->qs));
-        CK(cudaStreamWaitEvent(s, h->ev_qdone, 0));
+        CK(cudaEventRecord(h->ev_comb, h->qs));
+        if (sim) CK(cudaStreamWaitEvent(s, h->ev_comb, 0));  // k_sim_gemm reads Q_pc
         int64_t nsim = 0;  // k_sim_gemm launches
         if (!sedges.empty()) {  // A_pq <- Q_pc^T (A_pq Q_qc): all reads in the first launch, all writes in the second
           std::vector<SimGemm<T>> g1, g2;
