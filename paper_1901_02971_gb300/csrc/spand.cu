@@ -553,7 +553,9 @@ struct spand_handle_s {
   cudaEvent_t ev_comb = nullptr;  // the last k_form_q or k_combine launch
   unsigned apply_spin_limit = kBarrierSpins;  // polls per grid-barrier wait of the apply
   unsigned apply_bias = 0;                    // 1: failure-path test, no barrier completes
+  double* h_scal = nullptr;  // mapped host memory: the sums that the solve waits for
   ~spand_handle_s() {
+    if (h_scal) cudaFreeHost(h_scal);
     for (auto& a : aux)
       if (a) cudaStreamDestroy(a);
     if (qs) cudaStreamDestroy(qs);
@@ -3833,6 +3835,10 @@ int spand_solve(spand_handle h, const double* b, double* x, int32_t* iters, doub
   apply_autotune(h, z, s);
   double* part = V + 7 * n;
   double* sc = part + RED_BLOCKS;  // scalars
+  unsigned* count = (unsigned*)(sc + 12);
+  if (!h->h_scal) CK(cudaHostAlloc((void**)&h->h_scal, 64, cudaHostAllocMapped));
+  double* hrr = nullptr;  // r.r, b.b or the true residual, as the device left it in host memory
+  CK(cudaHostGetDevicePointer((void**)&hrr, h->h_scal, 0));
   const bool bdev = is_device_ptr(b), xdev = is_device_ptr(x);
   CK(cudaMemcpyAsync(io, b, n * sizeof(double), bdev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
   const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, 4096);
@@ -3844,40 +3850,51 @@ int spand_solve(spand_handle h, const double* b, double* x, int32_t* iters, doub
   CKLAUNCH();
   h->prof.launches += 1;
   CK(cudaMemsetAsync(xv, 0, n * sizeof(double), s));
-  auto dot = [&](const double* a, const double* c, double* out) {
-    k_dot<<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, a, c, part);
+  CK(cudaMemsetAsync(count, 0, sizeof(unsigned), s));
+  // a thread per element (for A: 4 lanes per row, 4 rows each), no more blocks than fill the GPU
+  const unsigned gv = (unsigned)std::min<int64_t>((n + RED_THREADS - 1) / RED_THREADS, RED_BLOCKS);
+  auto dot = [&](const double* a, const double* c, double* out, double* host) {
+    k_dot<<<gv, RED_THREADS, 0, s>>>(n, a, c, DotOut{part, count, out, host});
     CKLAUNCH();
-    k_reduce<<<1, RED_THREADS, 0, s>>>(part, RED_BLOCKS, out);
-    CKLAUNCH();
-    h->prof.launches += 2;
+    h->prof.launches += 1;
   };
-  auto read = [&](const double* d) {
-    double v = 0;
-    CK(cudaMemcpyAsync(&v, d, sizeof(double), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    h->prof.flush();
-    return v;
+  auto residual = [&](const double* xx, double* rr) {  // rr = b - A xx, its square to the host
+    k_spmv_dot<true><<<gv, RED_THREADS, 0, s>>>(n, rp, ci, va, xx, bp, rr, DotOut{part, count, sc + 2, hrr});
+    CKLAUNCH();
+    h->prof.launches += 1;
   };
   const double pcg_bytes = (double)h->nnz * 12 + (double)(n + 1) * 8 + 9.0 * n * 8;
-  cudaEvent_t e0, e1, e2;
+  cudaEvent_t e0, e1, e2, e3;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   CK(cudaEventCreate(&e2));
+  CK(cudaEventCreate(&e3));
   double apply_ms = 0, spmv_ms = 0;
   int napply = 0;
+  bool timed = false;  // an apply's event pair has not been read yet
+  // waits for the stream and returns the sum that the last kernel left for the
+  // host; the applies are timed here too, without a wait of their own
+  auto read = [&]() {
+    CK(cudaStreamSynchronize(s));
+    h->prof.flush();
+    if (timed) {
+      float ms = 0;
+      CK(cudaEventElapsedTime(&ms, e0, e1));
+      apply_ms += ms;
+      ++napply;
+      timed = false;
+    }
+    return *(volatile double*)h->h_scal;
+  };
   auto precond = [&](const double* src, double* dst) {
     CK(cudaEventRecord(e0, s));
     apply_any(h, src, dst, s);
     CK(cudaEventRecord(e1, s));
-    CK(cudaEventSynchronize(e1));
-    float ms = 0;
-    CK(cudaEventElapsedTime(&ms, e0, e1));
-    apply_ms += ms;
-    ++napply;
+    timed = true;
   };
-  // sc: [0] rz, [1] pq, [2] rr, [3] rz_new, [4] bb
-  dot(bp, bp, sc + 4);
-  const double bnorm = std::sqrt(read(sc + 4));
+  // sc: [0], [3] rz, alternating; [1] pq; [2] rr; [4] bb
+  dot(bp, bp, sc + 4, hrr);
+  const double bnorm = std::sqrt(read());
   int it = 0;
   double rel = 0.0;
   const double tol = h->opts.tol;
@@ -3888,65 +3905,47 @@ int spand_solve(spand_handle h, const double* b, double* x, int32_t* iters, doub
     k_copy_vec<<<g, 256, 0, s>>>(n, bp, r);
     CKLAUNCH();
     h->prof.launches += 1;
-    precond(r, z);
-    k_copy_vec<<<g, 256, 0, s>>>(n, z, p);
-    CKLAUNCH();
     int irz = 0, irzn = 3;
-    dot(r, z, sc + irz);
+    auto restart = [&]() {  // p = z = M M^T r
+      precond(r, z);
+      k_copy_vec<<<g, 256, 0, s>>>(n, z, p);
+      CKLAUNCH();
+      h->prof.launches += 1;
+      dot(r, z, sc + irz, nullptr);
+    };
+    restart();
     while (it < maxit) {
       CK(cudaEventRecord(e2, s));
       const int pid = h->prof.begin(F_PCG, s);
-      k_spmv_dot<<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, rp, ci, va, p, q, part);
+      k_spmv_dot<false><<<gv, RED_THREADS, 0, s>>>(n, rp, ci, va, p, nullptr, q, DotOut{part, count, sc + 1, nullptr});
       CKLAUNCH();
-      h->prof.launches += 4;
-      k_reduce<<<1, RED_THREADS, 0, s>>>(part, RED_BLOCKS, sc + 1);
+      k_update_xr<<<gv, RED_THREADS, 0, s>>>(n, sc + irz, sc + 1, xv, r, p, q, DotOut{part, count, sc + 2, hrr});
       CKLAUNCH();
-      // alpha = rz / pq
-      if (irz != 0) {
-        k_copy_vec<<<1, 32, 0, s>>>(1, sc + irz, sc + 0);
-        CKLAUNCH();
-        h->prof.launches += 1;
-        irz = 0;
-        irzn = 3;
-      }
-      k_update_xr<<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, sc, xv, r, p, q, part);
-      CKLAUNCH();
-      k_reduce<<<1, RED_THREADS, 0, s>>>(part, RED_BLOCKS, sc + 2);
-      CKLAUNCH();
-      h->prof.end(pid, s, 2.0 * h->nnz + 6.0 * n, pcg_bytes, 4);
-      CK(cudaEventRecord(e1, s));
+      h->prof.launches += 2;
+      h->prof.end(pid, s, 2.0 * h->nnz + 6.0 * n, pcg_bytes, 2);
+      CK(cudaEventRecord(e3, s));
       ++it;
-      const double rr = read(sc + 2);
+      const double rr = read();
       {
         float ms = 0;
-        CK(cudaEventElapsedTime(&ms, e2, e1));
+        CK(cudaEventElapsedTime(&ms, e2, e3));
         spmv_ms += ms;
       }
       if (std::sqrt(rr) / bnorm <= tol) {
-        k_residual<<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, rp, ci, va, xv, bp, r);
-        CKLAUNCH();
-        h->prof.launches += 1;
-        dot(r, r, sc + 2);
-        if (std::sqrt(read(sc + 2)) / bnorm <= tol) break;
-        precond(r, z);
-        k_copy_vec<<<g, 256, 0, s>>>(n, z, p);
-        CKLAUNCH();
-        h->prof.launches += 1;
-        dot(r, z, sc + 0);
+        residual(xv, r);
+        if (std::sqrt(read()) / bnorm <= tol) break;
+        restart();
         continue;
       }
       precond(r, z);
-      dot(r, z, sc + irzn);
+      dot(r, z, sc + irzn, nullptr);
       k_update_p<<<g, 256, 0, s>>>(n, sc + irzn, sc + irz, z, p);
       CKLAUNCH();
       h->prof.launches += 1;
       std::swap(irz, irzn);
     }
-    k_residual<<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, rp, ci, va, xv, bp, q);
-    CKLAUNCH();
-    h->prof.launches += 1;
-    dot(q, q, sc + 2);
-    rel = std::sqrt(read(sc + 2)) / bnorm;
+    residual(xv, q);
+    rel = std::sqrt(read()) / bnorm;
   }
   k_permute<<<g, 256, 0, s>>>(n, perm, xv, io, 0);
   CKLAUNCH();
@@ -3957,6 +3956,7 @@ int spand_solve(spand_handle h, const double* b, double* x, int32_t* iters, doub
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   cudaEventDestroy(e2);
+  cudaEventDestroy(e3);
   if (iters) *iters = it;
   if (relres) *relres = rel;
   h->st.n_cg = it;
