@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace spand {
 
 constexpr int TB = 64;    // tile edge of the factorization kernels
@@ -186,35 +188,66 @@ __device__ __forceinline__ void store_tile(const SqTileB<T, B>& s, T* P, int ld,
 
 // Upper Cholesky of the nb x nb diagonal tile s (A = U^T U, upper triangle
 // read and overwritten with U, lower triangle left as loaded) fused with the
-// inverse D = U^{-T} (lower, B x B, identity beyond nb).  Right-looking,
-// two pivot rows per step.  The owners of rows k and k + 1 of A and of D
-// publish them to shared memory; after a block barrier warp 0 alone forms
-// the 2 x 2 pivot block and the scaled rows (lane l takes the columns
-// l, l + 32, ...),
+// inverse D = U^{-T} (lower, B x B, identity beyond nb); B = 32.  Right-looking,
+// two pivot rows per step, 4 + 1 warps: warps 0-3 hold A and D in registers
+// (rows tx + PR a, columns ty + PC b), warp 4 forms the pivot rows (lane =
+// column),
 //   U_kk = sqrt(A_kk), U_k. = A_k. / U_kk,
 //   U_{k+1,k+1} = sqrt(A_{k+1,k+1} - U_{k,k+1}^2),
 //   U_{k+1,.} = (A_{k+1,.} - U_{k,k+1} U_k.) / U_{k+1,k+1},
 //   D_k. <- D_k. / U_kk,  D_{k+1,.} <- (D_{k+1,.} - U_{k,k+1} D_k.) / U_{k+1,k+1},
-// and publishes them; after a second barrier every thread updates the
-// 4 x CB elements it holds in registers (rows tx + PR a, columns ty + PC b)
-// with the rank-2 terms:
+// and the holders apply the rank-2 terms:
 //   A_ij -= U_ki U_kj + U_{k+1,i} U_{k+1,j} (k + 1 < i <= j),
 //   D_i. -= U_ki D_k. + U_{k+1,i} D_{k+1,.} (i > k + 1)   (row ops of L^{-1}, L = U^T).
-// The pivot scalars and the row scalings are FP64 work that every warp
-// would otherwise repeat on its own sub-partition (on this GPU a warp-wide
-// FP64 instruction occupies a sub-partition for tens of cycles), so one warp
-// does them once: fewer FP64 instructions per step on the critical path and
-// in total.  The row and result buffers alternate with the step parity.
-// 1 / U_kk comes from one reciprocal square root.  Returns false (for every
-// thread) if a pivot is not positive; nothing is stored then.
+// The chain pivot rows -> update -> pivot rows is what bounds it (a warp-wide
+// FP64 instruction occupies a sub-partition for 64 cycles), so the holders update
+// the row block of rows k + 2, k + 3 first and publish them, and do the other
+// three row blocks while warp 4 works on the next pivots: the two sides meet on
+// named barriers (bars 1, 2: rows published; 3, 4: pivot rows formed; by step
+// parity), which also alternate the buffers.  With every warp waiting for the
+// whole update and the pivot rows formed by warp 0, k_potrf_diag took 38 us on
+// average over a 64^3 factorization, now 31 (pivot family 8.4 -> 7.7 ms).  1 / U_kk comes from one reciprocal square root.  Returns false
+// (for every thread) if a pivot is not positive; nothing is stored then.
+constexpr int POTRF_NT = 160;  // threads: 4 holder warps and the pivot warp
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_sync(int id, int n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
 template <typename T, int B>
 __device__ bool potrf_inv_tile(SqTileB<T, B>& s, SqTileB<T, B>& D, int nb) {
   using G = TileGeom<B>;
   constexpr int PR = G::PR, PC = G::PC, CB = G::CB;
-  __shared__ T rowA[2][2][B], rowD[2][2][B];        // raw rows k, k + 1
-  __shared__ T scU[2][2][B], scD[2][2][B];          // scaled rows of U and of D
-  __shared__ T scP[2][2];                           // U_kk, U_{k+1,k+1}
+  static_assert(B == 32 && G::NTH == POTRF_NT - 32, "one lane per column, four holder warps");
+  __shared__ T rowA[2][2][B], rowD[2][2][B];  // raw rows k, k + 1
+  __shared__ T scU[2][2][B], scD[2][2][B];    // pivot rows of U and of D
   __shared__ int okP[2];
+  if (threadIdx.x >= G::NTH) {  // the pivot warp
+    const int lane = threadIdx.x & 31;
+    for (int k = 0; k < nb; k += 2) {
+      const int par = (k >> 1) & 1;
+      const bool two = k + 1 < nb;
+      bar_sync(1 + par, POTRF_NT);
+      const T a00 = rowA[par][0][k];
+      const T r0 = rsqrt(a00);
+      const T v0 = rowA[par][0][lane] * r0, e0 = rowD[par][0][lane] * r0;
+      const T u01 = __shfl_sync(0xffffffffu, v0, (k + 1) & 31);
+      const T s11 = two ? fma(-u01, u01, rowA[par][1][(k + 1) & 31]) : T(1);
+      const T r1 = rsqrt(s11);
+      scU[par][0][lane] = v0;
+      scD[par][0][lane] = e0;
+      scU[par][1][lane] = two ? fma(-u01, v0, rowA[par][1][lane]) * r1 : T(0);
+      scD[par][1][lane] = two ? fma(-u01, e0, rowD[par][1][lane]) * r1 : T(0);
+      const bool ok = (a00 > T(0)) && (s11 > T(0));
+      if (lane == 0) okP[par] = ok;
+      bar_arrive(3 + par, POTRF_NT);
+      if (!ok) return false;
+    }
+    __syncthreads();
+    return true;
+  }
   const int tx = threadIdx.x % PR, ty = threadIdx.x / PR;
   T a[4][CB], d[4][CB];
 #pragma unroll
@@ -225,15 +258,12 @@ __device__ bool potrf_inv_tile(SqTileB<T, B>& s, SqTileB<T, B>& D, int nb) {
       a[p][q] = s.v[i][j];
       d[p][q] = (i == j) ? T(1) : T(0);
     }
-  for (int k = 0; k < nb; k += 2) {
+  auto publish = [&](int k) {  // owners of rows k, k + 1 (compile-time register indices)
     const int par = (k >> 1) & 1;
-    const bool two = k + 1 < nb;
-    const int k1 = two ? k + 1 : k;  // a single last row repeats row k (unused)
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {  // owners of rows k, k + 1 publish them (compile-time register indices)
-      const int i = tx + PR * p;
-      if (i == k || i == k1) {
-        const int w = i == k ? 0 : 1;
+    for (int p = 0; p < 4; ++p) {
+      const int w = tx + PR * p - k;
+      if (w == 0 || w == 1) {
 #pragma unroll
         for (int q = 0; q < CB; ++q) {
           rowA[par][w][ty + PC * q] = a[p][q];
@@ -241,35 +271,17 @@ __device__ bool potrf_inv_tile(SqTileB<T, B>& s, SqTileB<T, B>& D, int nb) {
         }
       }
     }
-    __syncthreads();
-    if (threadIdx.x < 32) {  // warp 0: the pivot block and the scaled rows
-      const T a00 = rowA[par][0][k];
-      const T r0 = rsqrt(a00), u00 = a00 * r0;
-      const T u01 = two ? rowA[par][0][k1] * r0 : T(0);
-      const T s11 = two ? rowA[par][1][k1] - u01 * u01 : T(1);
-      const T r1 = rsqrt(s11), u11 = s11 * r1;
-      for (int j = threadIdx.x; j < B; j += 32) {
-        const T v0 = rowA[par][0][j] * r0, e0 = rowD[par][0][j] * r0;
-        scU[par][0][j] = v0;
-        scD[par][0][j] = e0;
-        scU[par][1][j] = two ? (rowA[par][1][j] - u01 * v0) * r1 : T(0);
-        scD[par][1][j] = two ? (rowD[par][1][j] - u01 * e0) * r1 : T(0);
-      }
-      if (threadIdx.x == 0) {
-        scP[par][0] = u00;
-        scP[par][1] = u11;
-        okP[par] = (a00 > T(0)) && (s11 > T(0));
-      }
-    }
-    __syncthreads();
+    __syncwarp();
+    bar_arrive(1 + par, POTRF_NT);
+  };
+  publish(0);
+  for (int k = 0; k < nb; k += 2) {
+    const int par = (k >> 1) & 1, k1 = k + 1;
+    const bool two = k1 < nb;
+    __syncwarp();
+    bar_sync(3 + par, POTRF_NT);
     if (!okP[par]) return false;  // uniform: every thread reads the same flag
-    T u0i[4], u1i[4], u0j[CB], u1j[CB], d0[CB], d1[CB];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int ci = tx + PR * q;
-      u0i[q] = scU[par][0][ci];
-      u1i[q] = scU[par][1][ci];
-    }
+    T u0j[CB], u1j[CB], d0[CB], d1[CB];
 #pragma unroll
     for (int q = 0; q < CB; ++q) {
       const int cj = ty + PC * q;
@@ -278,38 +290,47 @@ __device__ bool potrf_inv_tile(SqTileB<T, B>& s, SqTileB<T, B>& D, int nb) {
       d0[q] = scD[par][0][cj];
       d1[q] = scD[par][1][cj];
     }
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
+    const int ps = (k + 2) / PR;  // the row block of rows k + 2, k + 3
+    auto update = [&](auto pc) {
+      constexpr int p = decltype(pc)::value;
       const int i = tx + PR * p;
-      if (i == k) {  // finalise row k of U and of D
+      const T u0 = scU[par][0][i], u1 = scU[par][1][i];
+      if (i > k1) {
+        // U's upper triangle and D's lower triangle: patches entirely on the
+        // other side of the diagonal are skipped (zero in D, unused in U), as
+        // are D's column blocks past k + 1, where rows k, k + 1 of D are zero
 #pragma unroll
         for (int q = 0; q < CB; ++q) {
           const int j = ty + PC * q;
-          if (j == k) a[p][q] = scP[par][0];
-          else if (j > k) a[p][q] = u0j[q];
+          if (!G::below(p, q) && j >= i) a[p][q] = fma(-u1, u1j[q], fma(-u0, u0j[q], a[p][q]));
+          if (!G::above(p, q) && PC * q <= k1) d[p][q] = fma(-u1, d1[q], fma(-u0, d0[q], d[p][q]));
+        }
+      } else if (i == k) {  // finalise row k of U and of D
+#pragma unroll
+        for (int q = 0; q < CB; ++q) {
+          if (ty + PC * q >= k) a[p][q] = u0j[q];
           d[p][q] = d0[q];
         }
       } else if (two && i == k1) {  // finalise row k + 1
 #pragma unroll
         for (int q = 0; q < CB; ++q) {
-          const int j = ty + PC * q;
-          if (j == k1) a[p][q] = scP[par][1];
-          else if (j > k1) a[p][q] = u1j[q];
+          if (ty + PC * q >= k1) a[p][q] = u1j[q];
           d[p][q] = d1[q];
         }
-      } else if (i > k1) {
-        // U's upper triangle and D's lower triangle: patches entirely on the
-        // other side of the diagonal are skipped (they are zero in D and
-        // unused in U); D's entries above the diagonal stay zero because
-        // rows k, k + 1 of D are zero there
-#pragma unroll
-        for (int q = 0; q < CB; ++q) {
-          const int j = ty + PC * q;
-          if (!G::below(p, q) && j >= i) a[p][q] = fma(-u1i[p], u1j[q], fma(-u0i[p], u0j[q], a[p][q]));
-          if (!G::above(p, q)) d[p][q] = fma(-u1i[p], d1[q], fma(-u0i[p], d0[q], d[p][q]));
-        }
       }
+    };
+    auto each = [&](bool next) {
+      if ((ps == 0) == next) update(std::integral_constant<int, 0>{});
+      if ((ps == 1) == next) update(std::integral_constant<int, 1>{});
+      if ((ps == 2) == next) update(std::integral_constant<int, 2>{});
+      if ((ps == 3) == next) update(std::integral_constant<int, 3>{});
+    };
+    if (k + 2 < nb) {
+      each(true);
+      publish(k + 2);
     }
+    each(false);
+    if (k + 2 >= nb && ps < 4) each(true);  // no rows were published: the block that would have been first
   }
 #pragma unroll
   for (int p = 0; p < 4; ++p)

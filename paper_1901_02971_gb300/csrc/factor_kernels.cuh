@@ -99,7 +99,7 @@ __global__ void k_assemble(const double* __restrict__ vals, const int32_t* __res
 // Tile step k, phase 1: factor diagonal tile (k, k) of every block and store
 // the inverse of its factor, U_kk^{-T}, for the tile solves of phase 2.
 template <typename T, int B = TB>
-__global__ void __launch_bounds__(TileGeom<B>::NTH) k_potrf_diag(const RowDesc<T>* __restrict__ rows, int k,
+__global__ void __launch_bounds__(POTRF_NT) k_potrf_diag(const RowDesc<T>* __restrict__ rows, int k,
                                                                  int* info) {
   extern __shared__ __align__(16) unsigned char smraw[];
   SqTileB<T, B>& s = *reinterpret_cast<SqTileB<T, B>*>(smraw);
@@ -110,14 +110,16 @@ __global__ void __launch_bounds__(TileGeom<B>::NTH) k_potrf_diag(const RowDesc<T
   if (k0 >= d.n) return;
   const int nb = min(B, d.n - k0);
   T* P = d.R + k0 + (size_t)k0 * d.ld;
-  load_tile(s, P, d.ld, nb, nb);
+  if (threadIdx.x < TileGeom<B>::NTH) load_tile(s, P, d.ld, nb, nb);
   __syncthreads();
   if (!potrf_inv_tile(s, Id, nb)) {
     if (threadIdx.x == 0) atomicCAS(info, 0, (int)blockIdx.x + 1);
     return;
   }
-  store_tile(s, P, d.ld, nb, nb);
-  store_tile(Id, d.dinv + (size_t)k * B * B, B, B, B);
+  if (threadIdx.x < TileGeom<B>::NTH) {
+    store_tile(s, P, d.ld, nb, nb);
+    store_tile(Id, d.dinv + (size_t)k * B * B, B, B, B);
+  }
   pdl_trigger();
 }
 
@@ -342,13 +344,14 @@ __global__ void __launch_bounds__(INV_NT) k_inv_diag(const RowDesc<T>* __restric
     const int i = e & (TB - 1), j = e / TB;
     U.v[i][j] = (i < nb && j < nb) ? d.R[(k0 + i) + (size_t)(k0 + j) * d.ld] : (i == j ? T(1) : T(0));
   }
-  __syncthreads();
-  if (d.dinv32) {
+  if (d.dinv32)
+#pragma unroll 4
     for (int e = tid; e < 2 * 32 * 32; e += INV_NT) {
       const int h = e >> 10, i = (e >> 5) & 31, j = e & 31, o = 32 * h;  // tile h, entry (j, i) of U_bb^{-T}
       D.v[o + i][o + j] = o < nb ? (T)d.dinv32[((size_t)(2 * blockIdx.x + h) << 10) + (size_t)(32 * i + j)] : T(i == j);
     }
-  } else if (warp < 2) {  // D_bb = U_bb^{-1}: column j = lane, rows i <= j
+  __syncthreads();
+  if (!d.dinv32 && warp < 2) {  // D_bb = U_bb^{-1}: column j = lane, rows i <= j
     const int o = 32 * warp, j = lane;
     const T rinv = T(1) / U.v[o + lane][o + lane];
     T x[32];

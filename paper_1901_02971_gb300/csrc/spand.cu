@@ -711,7 +711,7 @@ static void potrf_batch(spand_handle h, const std::vector<RowDesc<T>>& rows, int
   int64_t nl = 0;
   for (int k = 0; k < nt; ++k) {
     nl += (nt - k - 1 > 0) ? 3 : 1;
-    launch_pdl(k_potrf_diag<T, B>, dim3(nb), dim3(nth), sm1, s, dr, k, d_info);
+    launch_pdl(k_potrf_diag<T, B>, dim3(nb), dim3(POTRF_NT), sm1, s, dr, k, d_info);
     const int m = nt - k - 1;
     if (m > 0) {
       launch_pdl(k_potrf_trsm<T, B>, dim3(m, nb), dim3(nth), sm2, s, dr, k);
