@@ -68,6 +68,10 @@ constexpr size_t kSmemPerSM = 228 * 1024;        // shared memory of one SM (eac
 constexpr int kCpqrMaxCluster = 8;              // thread-block cluster size (broadcasts to 16 CTAs cost 3.5x more)
 constexpr double kCqFp64Work = 2000;              // see its use
 constexpr size_t kGramBytes = size_t(4) << 30;    // most workspace for the separators' G blocks of a step
+// Descriptors up to this size are not copied to the device.  A call at limits of
+// 0 / 2 / 8 / 64 KB: 64 x 64 4.41 / 4.13 / 4.08 / 4.08 ms, extruded mesh 5.69 /
+// 5.50 / 5.42 / 5.33, 64^3 TF32 37.8 / 37.7 / 37.7 / 37.5; no limit gains nothing more.
+constexpr size_t kInPlaceBytes = 65536;
 constexpr int kAuxStreams = 8;
 constexpr double kCombineWork = 2e9;      // n^2 m of a step's separators up to which their G blocks are formed (FP32)
 constexpr double kApplyStreamBytes = 2e7;  // factor bytes of a phase of the apply from which it is LA_STREAM
@@ -554,7 +558,12 @@ struct spand_handle_s {
   unsigned apply_spin_limit = kBarrierSpins;  // polls per grid-barrier wait of the apply
   unsigned apply_bias = 0;                    // 1: failure-path test, no barrier completes
   double* h_scal = nullptr;  // mapped host memory: the sums that the solve waits for
+  std::vector<cudaEvent_t> step_ev;       // StepTimer
+  cudaEvent_t solve_ev[4] = {};           // the solve's timing
   ~spand_handle_s() {
+    for (auto& e : step_ev) cudaEventDestroy(e);
+    for (auto& e : solve_ev)
+      if (e) cudaEventDestroy(e);
     if (h_scal) cudaFreeHost(h_scal);
     for (auto& a : aux)
       if (a) cudaStreamDestroy(a);
@@ -661,6 +670,17 @@ static void* upload(spand_handle h, const Packer& pk, cudaStream_t s) {
   return d;
 }
 
+// The same for descriptors that only kernels on s read, before the stage's next
+// reset: small ones are left in the pinned staging memory, which the GPU reads
+// over its link to the host, and the copy in the stream is saved.
+template <typename T>
+static void* in_place(spand_handle h, const Packer& pk, cudaStream_t s) {
+  if (pk.empty() || pk.size > kInPlaceBytes) return upload<T>(h, pk, s);
+  void* src = h->stage.take(pk.size);
+  pk.write(src);
+  return src;
+}
+
 template <typename X>
 static X* at(void* base, size_t off) { return reinterpret_cast<X*>((char*)base + off); }
 
@@ -691,7 +711,7 @@ static void potrf_batch(spand_handle h, const std::vector<RowDesc<T>>& rows, int
   if (rows.empty()) return;
   Packer pk;
   size_t o = pk.add(rows);
-  void* d = upload<T>(h, pk, s);
+  void* d = in_place<T>(h, pk, s);
   const RowDesc<T>* dr = at<const RowDesc<T>>(d, o);
   int nmax = 0;
   for (auto& r : rows) nmax = std::max(nmax, r.n);
@@ -729,7 +749,7 @@ static void inv_diag_batch(spand_handle h, const std::vector<RowDesc<T>>& rows, 
   if (rows.empty()) return;
   Packer pk;
   size_t o = pk.add(rows);
-  void* d = upload<T>(h, pk, s);
+  void* d = in_place<T>(h, pk, s);
   int nmax = 0;
   for (auto& r : rows) nmax = std::max(nmax, r.n);
   const int nt = (nmax + TB - 1) / TB;
@@ -792,7 +812,7 @@ static void pivot_chol(spand_handle h, const std::vector<RowDesc<T>>& rows, int*
   if (wide && !cps.empty()) {
     Packer pk;
     const size_t oc = pk.add(cps);
-    void* d = upload<T>(h, pk, s);
+    void* d = in_place<T>(h, pk, s);
     dc = at<const PivotCopy>(d, oc);
     for (size_t b0 = 0; b0 < cps.size(); b0 += 65535) {
       const unsigned cnt = (unsigned)std::min<size_t>(cps.size() - b0, 65535);
@@ -804,7 +824,7 @@ static void pivot_chol(spand_handle h, const std::vector<RowDesc<T>>& rows, int*
   if (!bands.empty()) {
     Packer pk;
     const size_t ob = pk.add(bands);
-    void* d = upload<T>(h, pk, s);
+    void* d = in_place<T>(h, pk, s);
     const size_t sm = band_smem(bmax);
     ensure_smem((const void*)k_potrf_band<T>, sm);
     const int pid = h->prof.begin(F_POTRF, s);
@@ -840,7 +860,7 @@ static void trsm_batch(spand_handle h, const std::vector<TrsmTask<T>>& tasks, cu
   if (tasks.empty()) return;
   Packer pk;
   size_t o = pk.add(tasks);
-  void* d = upload<T>(h, pk, s);
+  void* d = in_place<T>(h, pk, s);
   const size_t sm = 2 * sizeof(SqTile<T>) + sizeof(TileSmem<T>);
   ensure_smem((const void*)k_trsm_cols<T>, sm);
   double fl = 0, by = 0;
@@ -951,7 +971,7 @@ static void copy_batch(spand_handle h, const std::vector<CopyTask<T>>& tasks_in,
   }
   Packer pk;
   size_t ot = pk.add(tasks), op = pk.add(tptr), oc = pk.add(cidx);
-  void* d = upload<T>(h, pk, s);
+  void* d = in_place<T>(h, pk, s);
   h->pool32.give(std::move(tptr));  // copied to pinned staging by upload
   h->pool32.give(std::move(cidx));
   double by = 0;
@@ -970,24 +990,25 @@ static void set_identity(spand_handle h, const std::vector<RowDesc<T>>& rows, cu
   if (rows.empty()) return;
   Packer pk;
   size_t o = pk.add(rows);
-  void* d = upload<T>(h, pk, s);
+  void* d = in_place<T>(h, pk, s);
   k_set_identity<T><<<dim3(8, (unsigned)rows.size()), 256, 0, s>>>(at<const RowDesc<T>>(d, o), (int)rows.size());
   CKLAUNCH();
   h->prof.launches += 1;
 }
 
 // Phase boundaries of every step (5 events per step, read once at the end of
-// the factorization, so that no step waits for its own timing).
+// the factorization, so that no step waits for its own timing); the handle
+// keeps the events.
 struct StepTimer {
-  std::vector<cudaEvent_t> ev;
-  explicit StepTimer(int nsteps) : ev(5 * (size_t)(nsteps + 1), nullptr) {
-    for (auto& e : ev) CK(cudaEventCreate(&e));
+  std::vector<cudaEvent_t>& ev;
+  StepTimer(std::vector<cudaEvent_t>& e, int nsteps) : ev(e) {
+    while (ev.size() < 5 * (size_t)(nsteps + 1)) {
+      cudaEvent_t x = nullptr;
+      CK(cudaEventCreate(&x));
+      ev.push_back(x);
+    }
   }
   cudaEvent_t at(int t, int k) const { return ev[5 * (size_t)t + k]; }
-  ~StepTimer() {
-    for (auto& e : ev)
-      if (e) cudaEventDestroy(e);
-  }
 };
 
 // Register-resident sparsification (FP32 factors): 512 threads per CTA, 64
@@ -2072,7 +2093,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
   stt.fail_step = 0;
   stt.fail_cluster = -1;
   HostScratch<T>& hs = h->template hs<T>();
-  StepTimer tm(L);
+  StepTimer tm(h->step_ev, L);
   h->stage.reset();  // the previous factorization ended with a stream synchronisation
   // non-positive pivot flags per step: [2t] elimination pivots, [2t+1]
   // scaling pivots ([0]: a bounded device wait gave up);
@@ -2087,9 +2108,12 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
   CK(cudaMemsetAsync(d_info, 0, ninfo * sizeof(int), s));
   std::vector<std::vector<int>> elim_cls(L + 1), scale_cls(L + 1);  // cluster of each pivot-batch entry
   std::vector<std::vector<std::vector<int>>> f_cls(L + 1);           // per step and colour: the f blocks' interfaces
-  auto check_pivots = [&](int upto) {  // after a stream synchronisation
-    std::vector<int> info(ninfo, 0);
-    CK(cudaMemcpy(info.data(), d_info, info.size() * sizeof(int), cudaMemcpyDeviceToHost));
+  int* info = nullptr;  // the flags as of the last readback
+  auto read_pivots = [&]() {  // before a stream synchronisation
+    info = (int*)h->stage.take(ninfo * sizeof(int));
+    CK(cudaMemcpyAsync(info, d_info, ninfo * sizeof(int), cudaMemcpyDeviceToHost, s));
+  };
+  auto check_pivots = [&](int upto) {  // after it (nothing has been staged since)
     if (info[0])
       throw Fail{SPAND_ERR_TIMEOUT, "Schur update: a bounded tensor-core wait (MMA completion or operand "
                                     "copy) timed out"};
@@ -2128,7 +2152,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
   {  // assemble A into the step-1 rows
     Packer pk;
     size_t orow = pk.add(lay.row);
-    void* d = upload<T>(h, pk, s);
+    void* d = in_place<T>(h, pk, s);
     const int64_t nnz = h->nnz;
     if (nnz > 0) {
       const int g = (int)std::min<int64_t>((nnz + 255) / 256, 4096);
@@ -2367,7 +2391,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         Packer pk;
         size_t ob = pk.add(blocks), oc = tma ? pk.add(flat_tma) : gram ? pk.add(gtask) : pk.add(flat), ot = pk.add(tiles);
         const size_t og = pk.add(gblock), op = pk.add(pulls), opt = pk.add(ptile);
-        void* d = upload<T>(h, pk, s);
+        void* d = in_place<T>(h, pk, s);
         double fl = 0, by = 0;
         for (auto& bl : blocks) {
           double ksum = 0;
@@ -2581,7 +2605,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       if (!sctl.empty()) {
         Packer pks;
         const size_t okt = pks.add(sct), okl = pks.add(sctl), okp = pks.add(scp);
-        void* dks = upload<T>(h, pks, s);
+        void* dks = in_place<T>(h, pks, s);
         double fl = 0;
         for (const ScaleTask<T>& k : sct) fl += (double)k.nq * k.nq * k.nc;
         const int pid = h->prof.begin(F_TRSM, s);
@@ -3009,6 +3033,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         run_pending();
         int32_t* hcur = (int32_t*)h->stage.take((size_t)n * sizeof(int32_t));
         CK(cudaMemcpyAsync(hcur, d_cur, (size_t)n * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        read_pivots();
         CK(cudaStreamSynchronize(s));
         std::copy(hcur, hcur + n, sz_after.begin());
         h->stage.reset();  // every copy issued so far has executed
@@ -3251,6 +3276,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
   }
   run_pending();
   if (h->ev_comb) CK(cudaStreamWaitEvent(s, h->ev_comb, 0));
+  read_pivots();
   CK(cudaStreamSynchronize(s));
   check_pivots(L);
   {
@@ -3864,11 +3890,9 @@ int spand_solve(spand_handle h, const double* b, double* x, int32_t* iters, doub
     h->prof.launches += 1;
   };
   const double pcg_bytes = (double)h->nnz * 12 + (double)(n + 1) * 8 + 9.0 * n * 8;
-  cudaEvent_t e0, e1, e2, e3;
-  CK(cudaEventCreate(&e0));
-  CK(cudaEventCreate(&e1));
-  CK(cudaEventCreate(&e2));
-  CK(cudaEventCreate(&e3));
+  for (auto& e : h->solve_ev)
+    if (!e) CK(cudaEventCreate(&e));
+  const cudaEvent_t e0 = h->solve_ev[0], e1 = h->solve_ev[1], e2 = h->solve_ev[2], e3 = h->solve_ev[3];
   double apply_ms = 0, spmv_ms = 0;
   int napply = 0;
   bool timed = false;  // an apply's event pair has not been read yet
@@ -3953,10 +3977,6 @@ int spand_solve(spand_handle h, const double* b, double* x, int32_t* iters, doub
   CK(cudaMemcpyAsync(x, io, n * sizeof(double), xdev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   check_apply(h);
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  cudaEventDestroy(e2);
-  cudaEventDestroy(e3);
   if (iters) *iters = it;
   if (relres) *relres = rel;
   h->st.n_cg = it;
