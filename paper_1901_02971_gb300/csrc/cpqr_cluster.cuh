@@ -644,8 +644,9 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
 
 // Q_pc = H_0 ... H_{r-1} [I_r; 0] (Sec. 2.6.1) of interfaces whose QR kernel
 // has finished, from the reflectors it left in V and tau and the rank in
-// cur_size[p] (or in the task's rank_out).  Launched per colour on a side stream, so that it overlaps the
-// next colour's QR; it is off the sparsification's critical path.  Block b of
+// cur_size[p] (or in the task's rank_out).  Launched on a side stream for a few
+// colours at a time, so that it overlaps the next colours' QR; it is off the
+// sparsification's critical path.  Block b of
 // an interface (nb blocks each) takes the column pairs (c, c + nb NW) with
 // c = b NW + warp (mod 2 nb NW), so every block meets chains of every length;
 // V is copied into shared memory when it fits (smem_elems elements).
