@@ -27,6 +27,8 @@
 
 #include <cooperative_groups.h>
 
+#include <cfloat>
+
 #include "dense_tiles.cuh"
 
 namespace spand {
@@ -89,6 +91,11 @@ __host__ __device__ inline int cq_ld(int np) {
 }
 
 template <typename T>
+struct CqMax {       // largest finite value
+  static constexpr T value = sizeof(T) == 4 ? T(FLT_MAX) : T(DBL_MAX);
+};
+
+template <typename T>
 struct CqShared {     // fixed part of the dynamic shared memory
   // pivot candidates, double-buffered by step parity (a fast warp or CTA
   // writes step k+1 while a slow one may still read step k): with C == 1 one
@@ -139,9 +146,14 @@ __device__ __forceinline__ void cq_warp_argmax(double& v, int& j) {
   j = __reduce_min_sync(0xffffffffu, hi == best && lo == bl ? j : INT_MAX);
   v = __hiloint2double(best, (int)bl);
 }
-// a > b for such values (squared norms, or -1)
-__device__ __forceinline__ bool cq_greater(float a, float b) { return __float_as_int(a) > __float_as_int(b); }
-__device__ __forceinline__ bool cq_greater(double a, double b) { return __double_as_longlong(a) > __double_as_longlong(b); }
+// a > b for such values (squared norms, or -1); a NaN (whose bit pattern lies
+// above infinity's) is never greater, so it is never a pivot
+__device__ __forceinline__ bool cq_greater(float a, float b) {
+  return __float_as_int(a) > __float_as_int(b) && __float_as_int(a) <= 0x7f800000;
+}
+__device__ __forceinline__ bool cq_greater(double a, double b) {
+  return __double_as_longlong(a) > __double_as_longlong(b) && __double_as_longlong(a) <= 0x7ff0000000000000LL;
+}
 __device__ __forceinline__ bool cq_live(float v) { return __float_as_int(v) >= 0; }
 __device__ __forceinline__ bool cq_live(double v) { return __double2hiint(v) >= 0; }
 
@@ -593,7 +605,10 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
       if constexpr (VW == 4) dot = ((a0 + b0) + (a1 + b1)) + ((a2 + b2) + (a3 + b3));
       else dot = (a0 + b0) + (a1 + b1);
       dot = cq_group_sum<LG>(dot);
-      const T ws = gam * dot;
+      T ws = gam * dot;
+      // |R_kk|^2 below the reciprocal's range (an almost decoupled interface):
+      // gam = -1 / (beta amb) overflows, the two divisions do not
+      if (gam > CqMax<T>::value) ws = -(dot / (pcol[k] - amb)) / amb;
       T q0 = 0, q1 = 0, q2 = 0, q3 = 0;
       if (lg == 0) {  // rows > k enter the norm
         xk.x = fma(-ws, pk.x, xk.x);
