@@ -664,7 +664,8 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
 // sparsification's critical path.  Block b of
 // an interface (nb blocks each) takes the column pairs (c, c + nb NW) with
 // c = b NW + warp (mod 2 nb NW), so every block meets chains of every length;
-// V is copied into shared memory when it fits (smem_elems elements).
+// V is copied into shared memory when it fits beside the rank's tau, which
+// always does (smem_elems elements in all).
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT) k_form_q(const CpqrTask<T>* __restrict__ tasks,
                                                  const int32_t* __restrict__ list,

@@ -1283,7 +1283,8 @@ static std::vector<int> sparsify_randomized(spand_handle h, int t, const std::ve
         for (int k : alist) {
           const int km = std::min(rt[k].np, ub[k]);
           kmx = std::max(kmx, km);
-          need = std::max(need, align256((size_t)km * sizeof(T)) + (size_t)rt[k].np * km * sizeof(T));
+          // tau takes the rank, which is np where no column is left to compress against
+          need = std::max(need, align256((size_t)rt[k].np * sizeof(T)) + (size_t)rt[k].np * km * sizeof(T));
         }
         const size_t qsm = std::min(need + 256, (size_t)227 * 1024);
         const int nb = std::max(1, (kmx + 2 * NWQ - 1) / (2 * NWQ));
@@ -2949,7 +2950,8 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
               const CpqrTask<T>& tk = tasks[list[li]];
               const int km = std::min(tk.np, tk.m_max);
               kmx = std::max(kmx, km);
-              need = std::max(need, align256((size_t)km * sizeof(T)) + (size_t)tk.np * km * sizeof(T));
+              // tau takes the rank, which is np where no column is left to compress against
+              need = std::max(need, align256((size_t)tk.np * sizeof(T)) + (size_t)tk.np * km * sizeof(T));
             }
             const size_t qsm = std::min(need + 256, (size_t)227 * 1024);
             const int nb = std::max(1, (kmx + 2 * NWQ - 1) / (2 * NWQ));

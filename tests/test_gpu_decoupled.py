@@ -1,0 +1,47 @@
+"""Systems whose pattern holds stored zeros, so that interfaces have nothing (or
+nothing left) to be compressed against: some are cut to rank 0, and those whose
+neighbours are all gone are kept whole, wider than their coupling.  x is compared
+with a sparse direct solve; with the preconditioner exact up to the factor's
+precision, the solve takes a few iterations.  Tolerance: the solve stops at a
+relative residual of 1e-12 and the condition numbers here are below 1e3."""
+import numpy as np
+import pytest
+import scipy.sparse.linalg as sla
+
+from paper_1901_02971_gb300 import Solver
+from paper_1901_02971_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(dim, n, part):
+    """The grid Laplacian with stored zeros in place of the couplings of every
+    unknown ("all") or of those in the lower half of the first coordinate."""
+    p = I.laplacian_2d(n) if dim == 2 else I.laplacian_3d(n)
+    rows = np.repeat(np.arange(p.n), np.diff(p.rowptr))
+    off = rows != p.colind
+    if part == "half":
+        low = np.asarray(p.coords)[:, 0] < n // 2
+        off &= low[rows] | low[p.colind]
+    p.vals = np.where(off, 0.0, p.vals)
+    return p
+
+
+@pytest.mark.parametrize("part", ["all", "half"])
+@pytest.mark.parametrize("order", ["coloured", "simultaneous"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "tf32"])
+@pytest.mark.parametrize("dim,n,levels", [(2, 33, 6), (3, 16, 4), (3, 21, 6)])
+def test_decoupled_interfaces(cuda_ok, dim, n, levels, precision, order, part):
+    import torch
+    p = _problem(dim, n, part)
+    b = I.rhs(p.n, 6)
+    ref = sla.spsolve(p.to_scipy().tocsc(), b)
+    s = Solver.from_problem(p, levels=levels, eps=1e-3, tol=1e-12, precision=precision, sparsify_order=order)
+    try:
+        s.factorize()
+        x, it, rr = s.solve(torch.from_numpy(b).cuda())
+        x = x.cpu().numpy()
+    finally:
+        s.close()
+    assert rr <= 1e-12 and it <= (3 if part == "all" else 20)
+    assert np.linalg.norm(x - ref) <= 1e-9 * np.linalg.norm(ref)
