@@ -281,8 +281,10 @@ __global__ void k_rand_decide(RandTask<T>* __restrict__ tasks, int n, double eps
 // into p's row and its transposes into the neighbours' rows, A_cc = I, the
 // size of p (no other task of the colour reads it: the interfaces of one
 // colour are not adjacent); a task with nothing to compress against keeps
-// p whole with Q_pc = I.  The warps of a task's CTAs take columns, the
-// lanes rows.
+// p whole with Q_pc = I (rank np), and one whose coupling is zero keeps its
+// first r dofs (its sketch has no reflectors, so Q was not formed; the blocks
+// are zero and the diagonal is I already).  The warps of a task's CTAs take
+// columns, the lanes rows.
 template <typename T>
 __global__ void __launch_bounds__(256) k_rand_writeback(const RandTask<T>* __restrict__ tasks,
                                                         const CpqrNbr<T>* __restrict__ nbrs,
@@ -292,13 +294,13 @@ __global__ void __launch_bounds__(256) k_rand_writeback(const RandTask<T>* __res
   const int gw = blockIdx.x * 8 + (threadIdx.x >> 5), nw = gridDim.x * 8;
   const int np = d.np;
   const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
-  if (d.m == 0 || np == 0) {
-    for (int c = gw; c < np; c += nw)
+  const int r = d.rank;
+  if (d.m == 0 || np == 0 || d.res[np + 1] == 0ull) {
+    for (int c = gw; c < r; c += nw)
       for (int i = lane; i < np; i += 32) d.Qc[i + (size_t)c * np] = (i == c) ? T(1) : T(0);
-    if (lead) cur_size[d.p] = np;
+    if (lead) cur_size[d.p] = r;
     return;
   }
-  const int r = d.rank;
   for (int j = gw; j < d.m; j += nw) {  // p's row
     T* dst = d.Rp + (size_t)d.tcol[j] * d.ldp;
     for (int i = lane; i < r; i += 32) dst[i] = d.W[i + (size_t)j * np];

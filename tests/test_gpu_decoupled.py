@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 import scipy.sparse.linalg as sla
 
+from oracle import spand_oracle as O
 from paper_1901_02971_gb300 import Solver
 from paper_1901_02971_gb300 import inputs as I
 
@@ -45,3 +46,36 @@ def test_decoupled_interfaces(cuda_ok, dim, n, levels, precision, order, part):
         s.close()
     assert rr <= 1e-12 and it <= (3 if part == "all" else 20)
     assert np.linalg.norm(x - ref) <= 1e-9 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("part", ["all", "half"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("dim,n,levels", [(2, 33, 6), (3, 16, 4)])
+def test_decoupled_interfaces_randomized(cuda_ok, dim, n, levels, precision, part):
+    """The sketch of a zero coupling is zero; its basis is then the identity's
+    columns (none of the rule's thresholds is met, so nothing is dropped), not
+    what the device memory held before.  Ranks equal to the oracle's in FP64."""
+    import torch
+    p = _problem(dim, n, part)
+    b = I.rhs(p.n, 6)
+    ref = sla.spsolve(p.to_scipy().tocsc(), b)
+    s = Solver.from_problem(p, levels=levels, eps=1e-3, tol=1e-12, precision=precision, compression="randomized")
+    try:
+        for size in (1 << 20, 1 << 24, 1 << 28):  # memory that was used before, and holds NaN
+            used = [torch.full((size // 8,), float("nan"), dtype=torch.float64, device="cuda") for _ in range(64 if size < 1 << 28 else 4)]
+            del used
+        torch.cuda.empty_cache()
+        s.factorize(p.vals)
+        ranks = [s.ranks(t)[1] for t in range(1, levels + 1)]
+        x, it, rr = s.solve(torch.from_numpy(b).cuda())
+        x = x.cpu().numpy()
+    finally:
+        s.close()
+    assert rr <= 1e-12 and it <= (3 if part == "all" else 20)
+    assert np.linalg.norm(x - ref) <= 1e-9 * np.linalg.norm(ref)
+    if precision == "fp64":
+        tree = O.analyze(p.n, p.rowptr, p.colind, p.coords, levels)
+        F = O.factorize(p.rowptr, p.colind, p.vals, tree, 1e-3, variant="OrthS-rand",
+                        sketch=lambda t, c, m, ell: O.sketch_philox(0, t, c, m, ell))
+        for t in range(1, levels + 1):
+            assert np.array_equal(ranks[t - 1], F.sizes_after[t - 1]), t
