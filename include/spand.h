@@ -178,8 +178,9 @@ int spand_analyze_batch(int32_t k, const spand_problem* probs, const spand_opts*
  * spand_factorize -- numeric factorization on the current CUDA device
  * (Algorithm 2).  vals: NULL to use the values given to spand_analyze, or a
  * new float64[nnz] array for the same pattern (host or device memory).
- * Errors: SPAND_ERR_NOT_SPD (spand_get_stats gives the failing step/cluster),
- * SPAND_ERR_CUDA, SPAND_ERR_OOM.  A failed factorization leaves the handle
+ * Errors: SPAND_ERR_NOT_SPD for a pivot block that is not positive definite or
+ * an interface whose coupling is not finite (spand_get_stats gives the failing
+ * step/cluster), SPAND_ERR_CUDA, SPAND_ERR_OOM.  A failed factorization leaves the handle
  * unfactorized.
  */
 int spand_factorize(spand_handle h, const double* vals, void* cuda_stream);

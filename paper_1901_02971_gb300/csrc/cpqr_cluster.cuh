@@ -56,6 +56,8 @@ struct CpqrTask {
   int32_t* rank_out;  // where the rank goes; nullptr: the cur_size array the sizes are read from
   int32_t p, np, ldp, nbeg, nend, m_max;
   int32_t nowb;       // 1: leave the blocks untouched (no W_cn write-back, simultaneous order)
+  int32_t id;         // the interface, as it is reported in bad
+  int32_t* bad;       // receives id + 1 if the coupling is not finite
 };
 
 // Destination of the rank of task d: a separate array when every interface of
@@ -65,6 +67,10 @@ template <typename T>
 __device__ __forceinline__ int32_t* cq_rank_dst(const CpqrTask<T>& d, int32_t* cur_size) {
   return d.rank_out ? d.rank_out : cur_size;
 }
+
+// Read from the task again: no register holds what only a failure needs.
+template <typename T>
+__device__ __noinline__ void cq_report(const CpqrTask<T>& d) { *d.bad = d.id + 1; }
 
 template <typename T>
 struct CqVec;
@@ -129,7 +135,9 @@ __host__ __device__ inline size_t cq_fixed_smem(int nnb, int np, int cols_per, i
 }
 
 // Warp-wide (largest value, lowest index on ties); every lane gets the result.
-// Values are squared norms (>= 0) or -1 for absent/retired columns.
+// Values are squared norms (>= 0, or a NaN without a sign) or -1 for
+// absent/retired columns.  The bit pattern of a NaN lies above infinity's, so a
+// column that holds one wins: the caller stops there and reports it.
 __device__ __forceinline__ void cq_warp_argmax(float& v, int& j) {
   // for floats >= 0 the signed-integer order of the bit patterns is the float
   // order, and every negative float is a negative integer
@@ -146,13 +154,16 @@ __device__ __forceinline__ void cq_warp_argmax(double& v, int& j) {
   j = __reduce_min_sync(0xffffffffu, hi == best && lo == bl ? j : INT_MAX);
   v = __hiloint2double(best, (int)bl);
 }
-// a > b for such values (squared norms, or -1); a NaN (whose bit pattern lies
-// above infinity's) is never greater, so it is never a pivot
-__device__ __forceinline__ bool cq_greater(float a, float b) {
-  return __float_as_int(a) > __float_as_int(b) && __float_as_int(a) <= 0x7f800000;
-}
-__device__ __forceinline__ bool cq_greater(double a, double b) {
-  return __double_as_longlong(a) > __double_as_longlong(b) && __double_as_longlong(a) <= 0x7ff0000000000000LL;
+// a > b for such values
+__device__ __forceinline__ bool cq_greater(float a, float b) { return __float_as_int(a) > __float_as_int(b); }
+__device__ __forceinline__ bool cq_greater(double a, double b) { return __double_as_longlong(a) > __double_as_longlong(b); }
+// infinity or NaN, and v without its sign (a sum of squares has one only as a
+// NaN), on the bit patterns: not work for the FP64 unit
+__device__ __forceinline__ bool cq_unbounded(float v) { return __float_as_int(v) >= 0x7f800000; }
+__device__ __forceinline__ bool cq_unbounded(double v) { return __double2hiint(v) >= 0x7ff00000; }
+__device__ __forceinline__ float cq_unsigned(float v) { return fabsf(v); }
+__device__ __forceinline__ double cq_unsigned(double v) {
+  return __hiloint2double(__double2hiint(v) & 0x7fffffff, __double2loint(v));
 }
 __device__ __forceinline__ bool cq_live(float v) { return __float_as_int(v) >= 0; }
 __device__ __forceinline__ bool cq_live(double v) { return __double2hiint(v) >= 0; }
@@ -302,7 +313,8 @@ __device__ __forceinline__ void cq_finish(const CpqrTask<T>& d, cg::cluster_grou
 //      into every CTA of the cluster; cluster barrier;
 //   2. every thread reduces the C candidates: pivot j*, |R_kk| = sqrt(norm)
 //      (norms are recomputed exactly each step); the truncation rule is
-//      checked here, uniformly;
+//      checked here, uniformly; a norm that is not finite ends the loop too,
+//      and is reported;
 //   3. the reflector H_k = I - gam u u^T from the raw pivot column p (read in
 //      place when C == 1, else from the copy its owner pushed), by every thread
 //      in FP32, by one warp in FP64;
@@ -449,7 +461,7 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
         if constexpr (VW == 4) s += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
         else s += x.x * x.x + x.y * x.y;
       }
-      nrm[c] = cq_group_sum<LG>(s);
+      nrm[c] = cq_unsigned(cq_group_sum<LG>(s));
     }
   }
 
@@ -511,7 +523,7 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
     auto reflector = [&]() {
       const T rkk = sqrt(gv > T(0) ? gv : T(0));
       if (k == 0) r00 = rkk;
-      stop = r00 == T(0) || rkk < eps * r00;
+      stop = r00 == T(0) || rkk < eps * r00 || cq_unbounded(gv);
       const T alpha = pcol[k];
       const T beta = alpha >= T(0) ? -rkk : rkk;
       amb = alpha - beta;
@@ -540,6 +552,7 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
       reflector();
     }
     if (stop) {
+      if (tid == 0 && cq_unbounded(gv)) cq_report(tasks[list[blockIdx.x / C]]);
       r = k;
       break;
     }

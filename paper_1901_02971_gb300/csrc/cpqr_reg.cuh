@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(NT, 1) k_cpqr_reg(const CpqrTask<T>* __restric
     // 1. the warp's candidate (largest trailing norm, lowest index); its group
     //    derives the reflector it would define and writes u into the warp's
     //    pivot slot (chunks below cbe; zeros above row k, alpha - beta at row k)
-    const bool live = own && nrm >= T(0);
+    const bool live = own && !(nrm < T(0));  // a NaN is live, and wins (cq_warp_argmax)
     int bj = live ? j0 + grp : INT_MAX;
     T bv = live ? nrm : T(-1);
     cq_warp_argmax(bv, bj);
@@ -407,7 +407,8 @@ __global__ void __launch_bounds__(NT, 1) k_cpqr_reg(const CpqrTask<T>* __restric
     if (gj == INT_MAX) gj = 0;  // unreachable: k < kmax <= m leaves a live column
     const T rkk = fabs(rec.b);
     if (k == 0) r00 = rkk;
-    if (r00 == T(0) || rkk < eps * r00) {
+    if (r00 == T(0) || rkk < eps * r00 || cq_unbounded(rkk)) {
+      if (tid == 0 && cq_unbounded(rkk)) cq_report(tasks[list[blockIdx.x / C]]);
       r = k;
       break;
     }

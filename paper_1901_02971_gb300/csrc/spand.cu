@@ -2097,7 +2097,8 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
   StepTimer tm(h->step_ev, L);
   h->stage.reset();  // the previous factorization ended with a stream synchronisation
   // non-positive pivot flags per step: [2t] elimination pivots, [2t+1]
-  // scaling pivots ([0]: a bounded device wait gave up);
+  // scaling pivots ([0]: a bounded device wait gave up; [1]: an interface whose
+  // coupling is not finite);
   // read at the next host synchronisation (the rank readback of a
   // sparsifying step, or the end of the factorization)
   // (then, for the interpolative variants, one flag per step and colour for
@@ -2134,6 +2135,11 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
                                             std::to_string(u)};
         }
       }
+    }
+    if (info[1]) {  // after the pivots: a pivot that failed leaves NaN behind
+      stt.fail_step = upto;
+      stt.fail_cluster = info[1] - 1;
+      throw Fail{SPAND_ERR_NOT_SPD, "interface coupling not finite at step " + std::to_string(upto)};
     }
   };
 
@@ -2678,6 +2684,8 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         tk.m_max = mm;
         tk.rank_out = d_rank;
         tk.nowb = sim ? 1 : 0;
+        tk.id = p;
+        tk.bad = d_info + 1;
         // smallest cluster whose per-CTA chunk fits in shared memory, and at
         // most ~2 columns per thread
         const size_t Lp = (size_t)cq_ld<T>(sz[p]);
