@@ -181,7 +181,7 @@ int spand_analyze_batch(int32_t k, const spand_problem* probs, const spand_opts*
  * Errors: SPAND_ERR_NOT_SPD for a pivot block that is not positive definite or
  * an interface whose coupling is not finite (spand_get_stats gives the failing
  * step/cluster), SPAND_ERR_CUDA, SPAND_ERR_OOM.  A failed factorization leaves the handle
- * unfactorized.
+ * unfactorized and nothing of it running on the device; the handle can be factorized again.
  */
 int spand_factorize(spand_handle h, const double* vals, void* cuda_stream);
 
@@ -370,6 +370,15 @@ int spand_set_apply_shape(spand_handle h, int32_t ctas_per_sm);
  *                 normal barriers.
  */
 int spand_set_apply_wait(spand_handle h, uint32_t polls, int32_t unreachable);
+
+/*
+ * spand_set_factor_fault -- failure-path knob (not part of the method).  The
+ * next spand_factorize on h ends with error `code` (SPAND_ERR_*), raised on the
+ * host once the elimination of step `step` (1-based) has been queued, so with
+ * kernels in flight; later calls are not affected.  step 0 takes it back; a step
+ * that the factorization does not reach leaves it standing.
+ */
+int spand_set_factor_fault(spand_handle h, int32_t step, int32_t code);
 
 void spand_destroy(spand_handle h);
 

@@ -43,7 +43,7 @@ EXPORTS = ["spand_default_opts", "spand_analyze", "spand_analyze_batch", "spand_
            "spand_get_tree", "spand_get_step", "spand_get_ranks", "spand_get_stats",
            "spand_get_phase_times", "spand_set_profiling", "spand_get_kernel_profile",
            "spand_reset_kernel_profile", "spand_get_launch_count", "spand_set_apply_wait", "spand_set_apply_shape",
-           "spand_destroy",
+           "spand_set_factor_fault", "spand_destroy",
            "spand_error_string",
            "spand_last_error"]
 KERNEL_FAMILIES = ["potrf", "trsm", "schur", "cpqr", "copy", "apply", "pcg"]
@@ -109,6 +109,7 @@ def lib():
     L.spand_get_launch_count.argtypes = [C.c_void_p, C.POINTER(C.c_int64)]
     L.spand_set_apply_wait.argtypes = [C.c_void_p, C.c_uint32, C.c_int32]
     L.spand_set_apply_shape.argtypes = [C.c_void_p, C.c_int32]
+    L.spand_set_factor_fault.argtypes = [C.c_void_p, C.c_int32, C.c_int32]
     L.spand_destroy.argtypes = [C.c_void_p]
     L.spand_destroy.restype = None
     L.spand_error_string.argtypes = [C.c_int]
@@ -302,6 +303,12 @@ def spand_set_apply_wait(h: int, polls: int = 0, unreachable: bool = False):
 def spand_set_apply_shape(h: int, ctas_per_sm: int = 0):
     """CTAs per SM of the preconditioner apply (1..4), or 0: autotuned."""
     _check(lib().spand_set_apply_shape(h, ctas_per_sm))
+
+
+def spand_set_factor_fault(h: int, step: int, code: int = SPAND_ERR_STATE):
+    """Failure-path knob: the next factorization fails on the host with `code`
+    after it has queued the elimination of `step` (0 takes it back)."""
+    _check(lib().spand_set_factor_fault(h, step, code))
 
 
 def spand_destroy(h: int):

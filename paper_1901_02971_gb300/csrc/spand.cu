@@ -49,9 +49,11 @@ struct Fail {
 #define CK(expr)                                                                              \
   do {                                                                                        \
     cudaError_t e_ = (expr);                                                                  \
-    if (e_ != cudaSuccess)                                                                    \
+    if (e_ != cudaSuccess) {                                                                  \
+      cudaGetLastError(); /* or the next launch check would report this error again */       \
       throw Fail{e_ == cudaErrorMemoryAllocation ? SPAND_ERR_OOM : SPAND_ERR_CUDA,            \
                  std::string(#expr) + ": " + cudaGetErrorString(e_)};                         \
+    }                                                                                         \
   } while (0)
 
 #define CKLAUNCH() CK(cudaGetLastError())
@@ -557,6 +559,7 @@ struct spand_handle_s {
   cudaEvent_t ev_comb = nullptr;  // the last k_form_q or k_combine launch
   unsigned apply_spin_limit = kBarrierSpins;  // polls per grid-barrier wait of the apply
   unsigned apply_bias = 0;                    // 1: failure-path test, no barrier completes
+  int fault_step = 0, fault_code = 0;         // failure-path test: the next factorization fails on the host here
   double* h_scal = nullptr;  // mapped host memory: the sums that the solve waits for
   std::vector<cudaEvent_t> step_ev;       // StepTimer
   cudaEvent_t solve_ev[4] = {};           // the solve's timing
@@ -658,6 +661,18 @@ static void ensure_streams(spand_handle h) {
   CK(cudaEventCreateWithFlags(&h->ev_comb, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
   for (auto& e : h->ev_join) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+}
+
+// Waits for everything a factorization on s has queued, its side streams
+// included.  A factorization that ends with an error does this before it
+// returns: kernels in flight read descriptors in the staging memory and write
+// the arenas, which the next one reuses, perhaps on another stream.
+static void quiesce(spand_handle h, cudaStream_t s) {
+  cudaStreamSynchronize(s);
+  for (cudaStream_t a : h->aux)
+    if (a) cudaStreamSynchronize(a);
+  if (h->qs) cudaStreamSynchronize(h->qs);
+  cudaGetLastError();
 }
 
 template <typename T>
@@ -2079,8 +2094,6 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
   const int L = tr.L;
   const double eps = h->opts.eps;
   const int skip = h->opts.skip;
-  // a failed factorization may have left work on the side stream
-  if (h->ev_comb) CK(cudaStreamWaitEvent(s, h->ev_comb, 0));
   h->persist.reset();
   h->descs.reset();
   std::vector<ApplyStep<T>> apply;
@@ -2095,7 +2108,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
   stt.fail_cluster = -1;
   HostScratch<T>& hs = h->template hs<T>();
   StepTimer tm(h->step_ev, L);
-  h->stage.reset();  // the previous factorization ended with a stream synchronisation
+  h->stage.reset();  // the previous factorization ended with a wait, also one that failed (quiesce)
   // non-positive pivot flags per step: [2t] elimination pivots, [2t+1]
   // scaling pivots ([0]: a bounded device wait gave up; [1]: an interface whose
   // coupling is not finite);
@@ -2231,6 +2244,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       if (h->splan.size() < (size_t)L + 1) h->splan.resize((size_t)L + 1);
       auto& plan = h->splan[t];
       if (!plan.built) {
+        plan = std::decay_t<decltype(plan)>();  // a failure may have left it half built
         std::unordered_map<int64_t, int32_t> bid;
         std::vector<std::vector<int32_t>> cl;  // per block: contribution triples (sep, ea, eb)
         for (int sidx : seps) {
@@ -2444,6 +2458,10 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
         h->prof.launches += gram ? 2 : 1;
         h->prof.end(pid, s, fl, by, gram ? 2 : 1);
       }
+    }
+    if (h->fault_step == t) {
+      h->fault_step = 0;
+      throw Fail{h->fault_code, "failure asked for at step " + std::to_string(t)};
     }
     CK(cudaEventRecord(tm.at(t, 1), s));
     // ------------------------------------------------ apply ops of the elimination
@@ -3134,6 +3152,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       if (h->mplan.size() < (size_t)L + 1) h->mplan.resize((size_t)L + 1);
       auto& mp = h->mplan[t];
       if (!mp.built) {
+        mp = std::decay_t<decltype(mp)>();
         mp.ptr.assign(1, 0);
         for (int a : rems) {
           const int P = pof[a];
@@ -3744,10 +3763,13 @@ int spand_factorize(spand_handle h, const double* vals, void* cuda_stream) {
     h->st.fail_step = 0;
     h->st.fail_cluster = -1;
     rc = SPAND_OK;
-  } else if (h->opts.precision == SPAND_FP64) {
-    rc = factorize_impl<double>(h, s);
   } else {
-    rc = factorize_impl<float>(h, s);
+    try {
+      rc = h->opts.precision == SPAND_FP64 ? factorize_impl<double>(h, s) : factorize_impl<float>(h, s);
+    } catch (...) {
+      quiesce(h, s);
+      throw;
+    }
   }
   h->fprec = h->opts.precision;
   CK(cudaStreamSynchronize(s));
@@ -4008,6 +4030,17 @@ int spand_set_apply_wait(spand_handle h, uint32_t polls, int32_t unreachable) {
   if (!h) { g_err = "null handle"; return SPAND_ERR_INVALID_ARG; }
   h->apply_spin_limit = polls ? polls : kBarrierSpins;
   h->apply_bias = unreachable ? 1u : 0u;
+  return SPAND_OK;
+}
+
+int spand_set_factor_fault(spand_handle h, int32_t step, int32_t code) {
+  if (!h) { g_err = "null handle"; return SPAND_ERR_INVALID_ARG; }
+  if (step < 0 || (step > 0 && (code <= SPAND_OK || code > SPAND_ERR_TIMEOUT))) {
+    g_err = "step must be >= 0 and code an error code";
+    return SPAND_ERR_INVALID_ARG;
+  }
+  h->fault_step = step;
+  h->fault_code = code;
   return SPAND_OK;
 }
 

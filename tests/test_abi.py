@@ -240,3 +240,19 @@ def test_variant_option(spand_lib):
         if h.value:
             L.spand_destroy(h.value)
         assert rc == want, (var, order, comp, rc)
+
+
+def test_factor_fault_knob_argument_checks(spand_lib):
+    """Host-side checks of spand_set_factor_fault."""
+    f = spand_lib.spand_set_factor_fault
+    assert f(None, 1, L.SPAND_ERR_STATE) == L.SPAND_ERR_INVALID_ARG
+    p = I.laplacian_2d(6)
+    h = L.spand_analyze(p.rowptr, p.colind, p.vals, p.coords, L.default_opts(levels=2))
+    try:
+        assert f(h, -1, L.SPAND_ERR_STATE) == L.SPAND_ERR_INVALID_ARG
+        assert f(h, 1, L.SPAND_OK) == L.SPAND_ERR_INVALID_ARG
+        assert f(h, 1, 99) == L.SPAND_ERR_INVALID_ARG
+        assert f(h, 1, L.SPAND_ERR_OOM) == L.SPAND_OK
+        assert f(h, 0, 0) == L.SPAND_OK
+    finally:
+        L.spand_destroy(h)
