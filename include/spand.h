@@ -182,6 +182,8 @@ int spand_analyze_batch(int32_t k, const spand_problem* probs, const spand_opts*
  * an interface whose coupling is not finite (spand_get_stats gives the failing
  * step/cluster), SPAND_ERR_CUDA, SPAND_ERR_OOM.  A failed factorization leaves the handle
  * unfactorized and nothing of it running on the device; the handle can be factorized again.
+ * Where device memory runs out, the call tries once more without the workspaces and
+ * factor blocks that only save time; SPAND_ERR_OOM means that this failed too.
  */
 int spand_factorize(spand_handle h, const double* vals, void* cuda_stream);
 
@@ -372,11 +374,27 @@ int spand_set_apply_shape(spand_handle h, int32_t ctas_per_sm);
 int spand_set_apply_wait(spand_handle h, uint32_t polls, int32_t unreachable);
 
 /*
+ * spand_set_factor_limits -- limits of the next factorizations on h (not part of
+ * the method).
+ *   workspace_bytes   : most device memory for the workspace with which the
+ *                       Schur update of a step takes a separator's couplings as
+ *                       one block (-1 = the default, 4 GiB, and never more than
+ *                       an eighth of the free memory; 0 = none: the update per
+ *                       pair of clusters, slower, equal up to rounding).
+ *   phases_per_launch : phases of the preconditioner apply per launch, 1..96
+ *                       (0 = the default, 96; z has the same bits for all).
+ */
+int spand_set_factor_limits(spand_handle h, int64_t workspace_bytes, int32_t phases_per_launch);
+
+/*
  * spand_set_factor_fault -- failure-path knob (not part of the method).  The
  * next spand_factorize on h ends with error `code` (SPAND_ERR_*), raised on the
  * host once the elimination of step `step` (1-based) has been queued, so with
  * kernels in flight; later calls are not affected.  step 0 takes it back; a step
- * that the factorization does not reach leaves it standing.
+ * that the factorization does not reach leaves it standing.  With
+ * SPAND_ERR_OOM the call itself goes on as it does when device memory runs out:
+ * it gives back the factorization's memory and starts again without the blocks
+ * that only save time, for the rest of the handle's life.
  */
 int spand_set_factor_fault(spand_handle h, int32_t step, int32_t code);
 

@@ -43,7 +43,7 @@ EXPORTS = ["spand_default_opts", "spand_analyze", "spand_analyze_batch", "spand_
            "spand_get_tree", "spand_get_step", "spand_get_ranks", "spand_get_stats",
            "spand_get_phase_times", "spand_set_profiling", "spand_get_kernel_profile",
            "spand_reset_kernel_profile", "spand_get_launch_count", "spand_set_apply_wait", "spand_set_apply_shape",
-           "spand_set_factor_fault", "spand_destroy",
+           "spand_set_factor_fault", "spand_set_factor_limits", "spand_destroy",
            "spand_error_string",
            "spand_last_error"]
 KERNEL_FAMILIES = ["potrf", "trsm", "schur", "cpqr", "copy", "apply", "pcg"]
@@ -110,6 +110,7 @@ def lib():
     L.spand_set_apply_wait.argtypes = [C.c_void_p, C.c_uint32, C.c_int32]
     L.spand_set_apply_shape.argtypes = [C.c_void_p, C.c_int32]
     L.spand_set_factor_fault.argtypes = [C.c_void_p, C.c_int32, C.c_int32]
+    L.spand_set_factor_limits.argtypes = [C.c_void_p, C.c_int64, C.c_int32]
     L.spand_destroy.argtypes = [C.c_void_p]
     L.spand_destroy.restype = None
     L.spand_error_string.argtypes = [C.c_int]
@@ -309,6 +310,12 @@ def spand_set_factor_fault(h: int, step: int, code: int = SPAND_ERR_STATE):
     """Failure-path knob: the next factorization fails on the host with `code`
     after it has queued the elimination of `step` (0 takes it back)."""
     _check(lib().spand_set_factor_fault(h, step, code))
+
+
+def spand_set_factor_limits(h: int, workspace_bytes: int = -1, phases_per_launch: int = 0):
+    """Limits of the next factorizations: bytes of the Schur update's workspace
+    (-1 = default, 0 = none), phases of the apply per launch (0 = default)."""
+    _check(lib().spand_set_factor_limits(h, workspace_bytes, phases_per_launch))
 
 
 def spand_destroy(h: int):

@@ -69,7 +69,13 @@ constexpr size_t kCpqrChunkBudget = 224 * 1024;  // shared memory per sparsifica
 constexpr size_t kSmemPerSM = 228 * 1024;        // shared memory of one SM (each resident CTA also reserves 1 KB)
 constexpr int kCpqrMaxCluster = 8;              // thread-block cluster size (broadcasts to 16 CTAs cost 3.5x more)
 constexpr double kCqFp64Work = 2000;              // see its use
-constexpr size_t kGramBytes = size_t(4) << 30;    // most workspace for the separators' G blocks of a step
+// Most workspace for the separators' G blocks of a step, and the share of the
+// free device memory that they may take where the buffer has to grow: the update
+// has a form without them, and memory that other handles or programs will want is
+// worth more than the time between the two.  Largest by step (64^3 FP64, 96^3
+// FP32, 128^3 FP32): 0.29, 0.54, 1.97 GB.
+constexpr size_t kGramBytes = size_t(4) << 30;
+constexpr int kGramShare = 8;
 // Descriptors up to this size are not copied to the device.  A call at limits of
 // 0 / 2 / 8 / 64 KB: 64 x 64 4.41 / 4.13 / 4.08 / 4.08 ms, extruded mesh 5.69 /
 // 5.50 / 5.42 / 5.33, 64^3 TF32 37.8 / 37.7 / 37.7 / 37.5; no limit gains nothing more.
@@ -79,6 +85,8 @@ constexpr double kCombineWork = 2e9;      // n^2 m of a step's separators up to 
 constexpr double kApplyStreamBytes = 2e7;  // factor bytes of a phase of the apply from which it is LA_STREAM
 constexpr int64_t kApplyFewItems = 2000;    // 8-row items up to which it is LA_FEW
 constexpr int kApplyCtasPerSm = 4;  // the most CTAs per SM the apply autotuner tries
+// Phases per launch of the apply at most (their descriptors take 72 KB of shared memory, three CTAs per SM).
+constexpr int kLevelMaxPhases = 96;
 
 // Chunked bump allocator over cudaMalloc; reset() keeps the chunks for reuse.
 class DevArena {
@@ -176,9 +184,25 @@ struct DevBuf {
       cap = 0;
     }
     size_t c = align256(std::max<size_t>(bytes + bytes / 4, 256));
-    CK(cudaMalloc(&p, c));
+    void* q = nullptr;
+    CK(cudaMalloc(&q, c));
+    p = q;
     cap = c;
     return p;
+  }
+  // The same for a use that can do without: nullptr (and no buffer) where it would
+  // have to grow beyond a share of the free memory, or cannot.
+  void* try_ensure(size_t bytes, int share) {
+    if (bytes <= cap && p) return p;
+    size_t avail = 0, total = 0;
+    CK(cudaMemGetInfo(&avail, &total));
+    if (bytes + bytes / 4 > (avail + cap) / share) return nullptr;
+    try {
+      return ensure(bytes);
+    } catch (const Fail& f) {
+      if (f.code != SPAND_ERR_OOM) throw;
+      return nullptr;
+    }
   }
   void release() {
     if (p) cudaFree(p);
@@ -560,6 +584,18 @@ struct spand_handle_s {
   unsigned apply_spin_limit = kBarrierSpins;  // polls per grid-barrier wait of the apply
   unsigned apply_bias = 0;                    // 1: failure-path test, no barrier completes
   int fault_step = 0, fault_code = 0;         // failure-path test: the next factorization fails on the host here
+  // A factorization ran out of device memory: from then on without the blocks
+  // that only save time (the separators' G_s and G_ns).
+  bool lean = false;
+  size_t gram_limit = kGramBytes;        // spand_set_factor_limits
+  int phase_limit = kLevelMaxPhases;     // the same: phases per launch of the next factorization's apply
+  int la_per_launch = kLevelMaxPhases;   // of the present one's
+  // Gives the device memory of the factorization back (nothing of it may be running).
+  void release_factor() {
+    persist.release();
+    descs.release();
+    for (DevBuf* b : {&scratch[0], &scratch[1], &d_piv64, &d_rand, &d_interp, &d_levels, &d_qc}) b->release();
+  }
   double* h_scal = nullptr;  // mapped host memory: the sums that the solve waits for
   std::vector<cudaEvent_t> step_ev;       // StepTimer
   cudaEvent_t solve_ev[4] = {};           // the solve's timing
@@ -1928,9 +1964,6 @@ static void add_level_step(spand_handle h, LevelProgram<T>& lp, int t, const std
   lp.steps.push_back(std::move(st));
 }
 
-// Phases per launch at most (their descriptors take 72 KB of shared memory, three CTAs per SM).
-constexpr int kLevelMaxPhases = 96;
-
 // The phases in execution order and the items of each.
 template <typename T>
 static void finish_level_program(spand_handle h, const LevelProgram<T>& lp, cudaStream_t s) {
@@ -1969,7 +2002,8 @@ static void finish_level_program(spand_handle h, const LevelProgram<T>& lp, cuda
   h->n_aprog = 0;
   const int np = h->n_lphase;
   const void* fn = (const void*)k_apply_levels<T>;
-  const size_t smem = la_smem<T>(std::min(np, kLevelMaxPhases));
+  h->la_per_launch = h->phase_limit;
+  const size_t smem = la_smem<T>(std::min(np, h->la_per_launch));
   ensure_smem(fn, smem + 1024);  // the kernel's static shared memory counts too
   int per_sm = 0;
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, LA_NT, smem));
@@ -2337,7 +2371,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
             tma = false;
         }
         // the separators' G (in the scratch buffer that step t + 1 will use),
-        // unless they would take more than kGramBytes, or BF16 operands
+        // unless they would take more than their limit, or BF16 operands
         size_t gbytes = 0;
         std::vector<size_t> goff(n, 0);
         for (int sidx : seps) {
@@ -2345,12 +2379,15 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
           goff[sidx] = gbytes;
           gbytes += align256(m * m * sizeof(T));
         }
-        const bool gram = gbytes <= kGramBytes && (!tc || tma);
+        const size_t glimit = h->lean ? 0 : h->gram_limit;
+        char* gbase = nullptr;
+        if (glimit > 0 && gbytes <= glimit && (!tc || tma))
+          gbase = (char*)h->scratch[(t + 1) & 1].try_ensure(gbytes, kGramShare);
+        const bool gram = gbase != nullptr;
         std::vector<GramTask<T>> gtask;
         std::vector<SchurBlock<T>> gblock;  // TF32: G as the target of k_schur_tma
         std::vector<PullContrib<T>>& pulls = hs.fresh(hs.pulls);
         std::vector<SchurTile>& ptile = hs.fresh(hs.ptile);
-        char* gbase = gram ? (char*)h->scratch[(t + 1) & 1].ensure(gbytes) : nullptr;
         const int ti = tc ? TC_M : TB, tj = tc ? TC_N : TB;
         if (gram) {
           for (int sidx : seps) {
@@ -2469,7 +2506,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
     if (levels) {
       double work = 0;
       for (int i : seps) work += (double)sz[i] * sz[i] * (lay.W[i] - sz[i]);
-      if (work <= kCombineWork / (sizeof(T) == 8 ? 20 : 1)) {
+      if (!h->lean && work <= kCombineWork / (sizeof(T) == 8 ? 20 : 1)) {
         gfac.assign(n, nullptr);
         std::vector<CombineTask<T>> gt;
         for (int i : seps) {
@@ -3340,9 +3377,9 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
 template <typename TF>
 static int launch_levels(spand_handle h, const LevelVecs<TF>& V, cudaStream_t s) {
   int nl = 0;
-  for (int p0 = 0; p0 < h->n_lphase; p0 += kLevelMaxPhases, ++nl) {
+  for (int p0 = 0; p0 < h->n_lphase; p0 += h->la_per_launch, ++nl) {
     const LevelPhase<TF>* ph = (const LevelPhase<TF>*)h->la_phases + p0;
-    int np = std::min(kLevelMaxPhases, h->n_lphase - p0);
+    int np = std::min(h->la_per_launch, h->n_lphase - p0);
     unsigned lim = h->apply_spin_limit, bias = h->apply_bias;
     unsigned* bar = (unsigned*)h->d_bar.p;
     int* err = (int*)h->d_bar.p + 2;
@@ -3764,8 +3801,19 @@ int spand_factorize(spand_handle h, const double* vals, void* cuda_stream) {
     h->st.fail_cluster = -1;
     rc = SPAND_OK;
   } else {
+    auto run = [&]() { return h->opts.precision == SPAND_FP64 ? factorize_impl<double>(h, s) : factorize_impl<float>(h, s); };
     try {
-      rc = h->opts.precision == SPAND_FP64 ? factorize_impl<double>(h, s) : factorize_impl<float>(h, s);
+      try {
+        rc = run();
+      } catch (const Fail& f) {  // out of device memory: once more with as little as it can do with
+        if (f.code != SPAND_ERR_OOM || h->lean) throw;
+        quiesce(h, s);
+        h->release_factor();
+        h->lean = true;
+        h->tmp_len = 0;
+        h->save_len = 0;
+        rc = run();
+      }
     } catch (...) {
       quiesce(h, s);
       throw;
@@ -4041,6 +4089,17 @@ int spand_set_factor_fault(spand_handle h, int32_t step, int32_t code) {
   }
   h->fault_step = step;
   h->fault_code = code;
+  return SPAND_OK;
+}
+
+int spand_set_factor_limits(spand_handle h, int64_t workspace_bytes, int32_t phases_per_launch) {
+  if (!h) { g_err = "null handle"; return SPAND_ERR_INVALID_ARG; }
+  if (workspace_bytes < -1 || phases_per_launch < 0 || phases_per_launch > kLevelMaxPhases) {
+    g_err = "workspace_bytes must be >= -1 and phases_per_launch in [0, 96]";
+    return SPAND_ERR_INVALID_ARG;
+  }
+  h->gram_limit = workspace_bytes < 0 ? kGramBytes : (size_t)workspace_bytes;
+  h->phase_limit = phases_per_launch ? phases_per_launch : kLevelMaxPhases;
   return SPAND_OK;
 }
 
