@@ -590,6 +590,15 @@ struct spand_handle_s {
   size_t gram_limit = kGramBytes;        // spand_set_factor_limits
   int phase_limit = kLevelMaxPhases;     // the same: phases per launch of the next factorization's apply
   int la_per_launch = kLevelMaxPhases;   // of the present one's
+  // Every device allocation of the handle: DevBuf members belong in this list.
+  size_t device_bytes() const {
+    size_t b = persist.bytes_held + descs.bytes_held;
+    for (const DevBuf* x :
+         {&scratch[0], &scratch[1], &d_vals, &d_asm_row, &d_asm_off, &d_prow, &d_pcol, &d_pval, &d_pval_src, &d_perm,
+          &d_vec, &d_tmp, &d_save, &d_piv64, &d_rand, &d_interp, &d_rowptr, &d_colind, &d_levels, &d_bar, &d_qc})
+      b += x->cap;
+    return b;
+  }
   // Gives the device memory of the factorization back (nothing of it may be running).
   void release_factor() {
     persist.release();
@@ -3822,8 +3831,6 @@ int spand_factorize(spand_handle h, const double* vals, void* cuda_stream) {
   h->fprec = h->opts.precision;
   CK(cudaStreamSynchronize(s));
   h->st.t_factor_s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-  h->st.device_bytes = (int64_t)(h->persist.bytes_held + h->descs.bytes_held + h->scratch[0].cap + h->scratch[1].cap +
-                                   h->d_piv64.cap);
   const size_t esz = h->fprec == SPAND_FP64 ? 8 : 4;
   h->st.apply_bytes = 2.0 * (double)h->st.mem_f * esz;
   h->factored = rc == SPAND_OK;
@@ -4234,6 +4241,7 @@ int spand_get_ranks(spand_handle h, int32_t t, int32_t* sizes_before, int32_t* s
 int spand_get_stats(spand_handle h, spand_stats* st) {
   if (!h || !st) { g_err = "null argument"; return SPAND_ERR_INVALID_ARG; }
   h->st.apply_ctas_per_sm = h->apply_ctas;
+  h->st.device_bytes = (int64_t)h->device_bytes();
   *st = h->st;
   return SPAND_OK;
 }
