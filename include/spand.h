@@ -62,8 +62,11 @@ enum {
                       in FP64 (on an FP64 copy of each pivot block, U and the
                       inverses of its diagonal tiles rounded to FP32);
                       triangular solves, Schur GEMMs, QR and the
-                      preconditioner apply in FP32; vectors, SpMV and the PCG
-                      recurrences in FP64 */
+                      preconditioner apply in FP32; the vectors it takes and
+                      returns, SpMV and the PCG recurrences in FP64 (inside the
+                      apply, values that products have formed are FP32; r and
+                      the sums of r and products, until a product reads them,
+                      OrthS: pairs of FP32 numbers, InS and In: FP64) */
   SPAND_TF32 = 2,  /* as SPAND_FP32, with the elimination's Schur GEMMs on the
                       tensor cores: TF32 operands, FP32 accumulation */
   SPAND_BF16 = 3   /* as SPAND_TF32 with BF16 operands (FP32 accumulation,
@@ -216,15 +219,18 @@ int spand_apply(spand_handle h, const double* r_dev, double* z_dev, void* cuda_s
  * acceptable.  The paper has no counterpart; this is a deployment variant.
  *   r_dev, z_dev : device float64[n], original ordering; they may alias.
  * Work space: one fixed array of 2^21 doubles (16 MiB) compiled into the
- * library, resident on every GPU that loads it until the process exits.  A
- * factorization whose apply needs more (n + its per-step temporaries + its
- * sparsification save area) is rejected with SPAND_ERR_INVALID_ARG before any
- * GPU work.  The first call on a device looks up that array's device address
+ * library, resident on every GPU that loads it until the process exits; the
+ * OrthS variant keeps n doubles there, its other work vectors belong to the
+ * handle (spand_factorize allocates them).  A factorization too large for the
+ * array (n + per-step temporaries + sparsification save area, which the
+ * interpolative variants keep there; the same limit holds for OrthS) is
+ * rejected with SPAND_ERR_INVALID_ARG before any GPU work.  The first call on a device looks up that array's device address
  * (cudaGetSymbolAddress), so make that first call before any stream capture.
  * All calls share the array and it keeps the last call's contents (nothing in
  * it needs to start at zero); calls whose GPU work overlaps -- on different
  * streams, handles or host threads -- race on it and must be serialised by the
- * caller.  Errors as spand_apply.
+ * caller (on one handle also with spand_apply and spand_solve).  Errors as
+ * spand_apply.
  */
 int spand_apply_noalloc(spand_handle h, const double* r_dev, double* z_dev, void* cuda_stream);
 
@@ -352,7 +358,8 @@ int spand_get_launch_count(spand_handle h, int64_t* launches);
  * library's autotuner choose at the first apply or solve after the handle's
  * first factorization, by timing every candidate on a scratch vector, and
  * keep that choice for the handle.  The shape never changes the result:
- * every item of an apply phase is computed by one CTA in a fixed order.
+ * every item of an apply phase is computed by one warp (interpolative variants:
+ * one CTA) in a fixed order.
  */
 int spand_set_apply_shape(spand_handle h, int32_t ctas_per_sm);
 

@@ -556,6 +556,9 @@ struct spand_handle_s {
   bool factored = false;
   std::vector<ApplyStep<double>> apply64;
   std::vector<ApplyStep<float>> apply32;
+  // doubles of per-step temporaries and of the save area: the work space of the
+  // interpolative variants' apply, and for every variant part of the size that
+  // spand_apply_noalloc is limited to
   int64_t tmp_len = 0, save_len = 0;
   spand_stats st{};
   double phase_ms[6] = {0, 0, 0, 0, 0, 0};
@@ -3426,7 +3429,7 @@ static void apply_levels(spand_handle h, const double* src, double* dst, cudaStr
   h->prof.end(pid, s, 0.0, h->st.apply_bytes, nl);
 }
 
-// tmp: h->tmp_len doubles of per-step temporaries; save: h->save_len doubles
+// Interpolative variants: tmp: h->tmp_len doubles of per-step temporaries; save: h->save_len doubles
 // of sparsification forward inputs (both scratch; nothing needs to start at 0).
 // One cooperative launch runs the whole apply program; a barrier timeout is
 // recorded in d_bar[2] and reported by check_apply().
@@ -3484,7 +3487,8 @@ static void apply_any(spand_handle h, const double* src, double* dst, cudaStream
 // the first apply after a handle's first factorization times 1 .. 4 CTAs per
 // SM (two applications each, on a scratch vector) and keeps the fastest for
 // the handle's later factorizations and solves.  Every item of a phase is
-// computed by one CTA in a fixed order whatever the grid, so the choice never
+// computed by one warp (interpolative variants: one CTA) in a fixed order
+// whatever the grid, so the choice never
 // changes a bit of z.  More CTAs stream the large leaf phases faster; fewer
 // make the grid barriers of many small phases cheaper.
 static void apply_autotune(spand_handle h, double* scratch, cudaStream_t s) {
@@ -3522,6 +3526,7 @@ static void apply_autotune(spand_handle h, double* scratch, cudaStream_t s) {
 static void ensure_solve_buffers(spand_handle h) {
   const int64_t n = std::max<int64_t>(h->n, 1);
   h->d_vec.ensure((size_t)(7 * n + RED_BLOCKS + 16) * sizeof(double));
+  if (h->opts.variant == SPAND_ORTHS) return;  // its apply works in d_levels
   h->d_tmp.ensure((size_t)std::max<int64_t>(h->tmp_len, 1) * sizeof(double));
   h->d_save.ensure((size_t)std::max<int64_t>(h->save_len, 1) * sizeof(double));
 }
@@ -3873,7 +3878,8 @@ int spand_apply(spand_handle h, const double* r_dev, double* z_dev, void* cuda_s
 // whole device memory pool (a framework's caching allocator with a fixed
 // budget), or a latency-critical loop where cudaMalloc / cudaFree would add
 // their implicit device-wide synchronisation.  spand_apply_noalloc computes the
-// same z = M M^T r with its work vectors in one fixed array that lives in the
+// same z = M M^T r with the vectors that spand_apply would allocate (beside
+// those that spand_factorize has allocated) in one fixed array that lives in the
 // library image itself (a static __device__ array, kNoAllocMaxDoubles doubles =
 // 16 MiB, resident on every GPU that loads the library until the process
 // exits), so the call itself never allocates.
