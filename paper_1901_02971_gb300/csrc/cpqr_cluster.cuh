@@ -27,8 +27,6 @@
 
 #include <cooperative_groups.h>
 
-#include <cfloat>
-
 #include "dense_tiles.cuh"
 
 namespace spand {
@@ -96,9 +94,14 @@ __host__ __device__ inline int cq_ld(int np) {
   return g * vw;
 }
 
+// Squared norms below this count as zero.  The interfaces' diagonal blocks are
+// the identity here, so a coupling of norm 1e-15 (FP64: 1e-145) is far below what
+// the factor's arithmetic resolves; and of smaller columns the squares lose
+// their digits to the end of the number range, so that a reflector formed from
+// them would be neither orthogonal nor, where its factor overflows, finite.
 template <typename T>
-struct CqMax {       // largest finite value
-  static constexpr T value = sizeof(T) == 4 ? T(FLT_MAX) : T(DBL_MAX);
+struct CqTiny {
+  static constexpr T value = sizeof(T) == 4 ? T(1e-30) : T(1e-290);
 };
 
 template <typename T>
@@ -521,7 +524,7 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
     T amb, gam;
     bool stop;
     auto reflector = [&]() {
-      const T rkk = sqrt(gv > T(0) ? gv : T(0));
+      const T rkk = gv < CqTiny<T>::value ? T(0) : sqrt(gv);
       if (k == 0) r00 = rkk;
       stop = r00 == T(0) || rkk < eps * r00 || cq_unbounded(gv);
       const T alpha = pcol[k];
@@ -618,10 +621,7 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
       if constexpr (VW == 4) dot = ((a0 + b0) + (a1 + b1)) + ((a2 + b2) + (a3 + b3));
       else dot = (a0 + b0) + (a1 + b1);
       dot = cq_group_sum<LG>(dot);
-      T ws = gam * dot;
-      // |R_kk|^2 below the reciprocal's range (an almost decoupled interface):
-      // gam = -1 / (beta amb) overflows, the two divisions do not
-      if (gam > CqMax<T>::value) ws = -(dot / (pcol[k] - amb)) / amb;
+      const T ws = gam * dot;
       T q0 = 0, q1 = 0, q2 = 0, q3 = 0;
       if (lg == 0) {  // rows > k enter the norm
         xk.x = fma(-ws, pk.x, xk.x);

@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(NT, 1) k_cpqr_reg(const CpqrTask<T>* __restric
         for (int u = 0; u < 8; ++u)
           if (c * 8 + u == qk) a = x[c * 8 + u];
         a = __shfl_sync(gmask, a, gbase + (k - qk * G));
-        const T rkk = sqrt(bv);
+        const T rkk = bv < CqTiny<T>::value ? T(0) : sqrt(bv);
         const T b = a >= T(0) ? -rkk : rkk;
         const T gam = rkk == T(0) ? T(0) : T(1) / (b * (b - a));
         const T amb = a - b;

@@ -46,3 +46,27 @@ def test_nan_is_an_error(cuda_ok, precision):
             s.factorize()
         finally:
             s.close()
+
+
+@pytest.mark.parametrize("order", ["coloured", "simultaneous"])
+@pytest.mark.parametrize("n,levels", [(12, 2), (16, 3), (21, 6)])
+@pytest.mark.parametrize("scale", [1e-13, 1e-16, 1e-18, 1e-19, 1e-20, 1e-22, 1e-24])
+def test_weak_couplings_fp32(cuda_ok, n, levels, scale, order):
+    """FP32 factors: squared column norms from 1e-27 down to beyond the subnormals.
+    The preconditioner is the inverse to FP32's precision, so the solve takes two
+    or three iterations to 1e-12."""
+    import torch
+    p = I.laplacian_3d(n)
+    rows = np.repeat(np.arange(p.n), np.diff(p.rowptr))
+    off = rows != p.colind
+    p.vals = np.where(off, p.vals * scale, p.vals)
+    s = Solver.from_problem(p, levels=levels, eps=1e-2, tol=1e-12, precision="fp32", sparsify_order=order).factorize()
+    try:
+        r = I.rhs(p.n, 5)
+        x, it, rr = s.solve(torch.from_numpy(r).cuda())
+        x = x.cpu().numpy()
+    finally:
+        s.close()
+    assert rr <= 1e-12 and it <= 3
+    # the residual of the stopping test, and the couplings themselves
+    assert np.abs(x * p.vals[~off] - r).max() <= 2e-12 * np.linalg.norm(r)
