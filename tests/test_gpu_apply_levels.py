@@ -62,3 +62,33 @@ def test_unscaled_steps_and_wide_couplings(cuda_ok, dim, n, levels, skip, precis
     u = 2.0 ** {"fp64": -53, "fp32": -24, "tf32": -11}[precision]
     err = np.linalg.norm(z - ref) / np.linalg.norm(ref)
     assert err <= 20 * _cond(dim, n) * u, err
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "tf32"])
+@pytest.mark.parametrize("dim,n,levels,skip", [(2, 33, 6, 2), (2, 65, 5, 1), (3, 13, 5, 2), (3, 17, 5, 0), (3, 21, 6, 3)])
+def test_unscaled_next_to_scaled_steps(cuda_ok, dim, n, levels, skip, precision):
+    """Steps whose clusters pass through unscaled (t <= skip) below scaled ones
+    (skip < t < levels), couplings of one to several tiles with ragged ends, on the
+    grid Laplacian plus 2 I (condition number at most 5 in 2D, 7 in 3D).  Bound:
+    20 cond u for the factors and products; TF32 operands of the Schur update add
+    2 * 2^-11 per step, times cond: at most 0.05, so that a missing or misplaced
+    contribution shows."""
+    import torch
+    assert skip + 1 < levels
+    p = I.laplacian_2d(n) if dim == 2 else I.laplacian_3d(n)
+    rows = np.repeat(np.arange(p.n), np.diff(p.rowptr))
+    p.vals = p.vals + np.where(rows == p.colind, 2.0, 0.0)
+    r = I.rhs(p.n, 4)
+    ref = sla.spsolve(p.to_scipy().tocsc(), r)
+    s = Solver.from_problem(p, levels=levels, eps=0.0, skip=skip, precision=precision).factorize()
+    try:
+        z = s.apply(torch.from_numpy(r).cuda()).cpu().numpy()
+    finally:
+        s.close()
+    cond = 1.0 + 2.0 * dim
+    tol = 20 * cond * 2.0 ** (-53 if precision == "fp64" else -24)
+    if precision == "tf32":
+        tol += 2 * levels * cond * 2.0 ** -11
+    assert tol < 0.1
+    err = np.linalg.norm(z - ref) / np.linalg.norm(ref)
+    assert err <= tol, err
