@@ -1476,6 +1476,7 @@ static std::vector<InterpOut<T>> sparsify_interp(spand_handle h, const std::vect
       d.ldp = tk.ldp;
       d.nbeg = tk.nbeg;
       d.nend = tk.nend;
+      d.bad = tk.bad;
       tcol_at[k] = tcol.size();
       for (int32_t e = tk.nbeg; e < tk.nend; ++e)
         for (int32_t jj = 0; jj < hsz[nbrs[e].q]; ++jj) tcol.push_back(nbrs[e].off_pq + jj);

@@ -48,7 +48,15 @@ struct InterpTask {
   T* XT;               // T_cf, r x nf, leading dimension r (factor storage)
   int32_t p, np, ldp, m, nbeg, nend;  // neighbours: nbrs[nbeg .. nend)
   int32_t r, nf, ldf, pad;            // set once the rank is known
+  int32_t* bad;        // receives p + 1 if the coupling is not finite
 };
+
+// Whether the remaining diagonal v (index j) goes before w (index i): the larger,
+// the lower index on ties; a NaN goes first, and is reported.
+__device__ __forceinline__ bool ip_before(double v, int j, double w, int i) {
+  if (v != v) return w == w || j < i;
+  return v > w || (v == w && j < i);
+}
 
 // G = A_np^T A_np: one 32 x 32 tile (ti <= tj) per CTA; tile lists are
 // (task, ti, tj).  Thread (ty, tx) computes rows 4 ty .. 4 ty + 3 of column
@@ -130,12 +138,12 @@ __global__ void __launch_bounds__(256) k_interp_factor(const InterpTask<T>* __re
     double bv = -1.0;
     int bj = INT_MAX;
     for (int i = tid; i < np; i += 256)
-      if (!used[i] && (dg[i] > bv || (dg[i] == bv && i < bj))) bv = dg[i], bj = i;
+      if (!used[i] && ip_before(dg[i], i, bv, bj)) bv = dg[i], bj = i;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
       const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
-      if (ov > bv || (ov == bv && oj < bj)) bv = ov, bj = oj;
+      if (ip_before(ov, oj, bv, bj)) bv = ov, bj = oj;
     }
     if (lane == 0) wv[warp] = bv, wj[warp] = bj;
     __syncthreads();
@@ -143,7 +151,7 @@ __global__ void __launch_bounds__(256) k_interp_factor(const InterpTask<T>* __re
       double v = wv[0];
       int j = wj[0];
       for (int w = 1; w < 8; ++w)
-        if (wv[w] > v || (wv[w] == v && wj[w] < j)) v = wv[w], j = wj[w];
+        if (ip_before(wv[w], wj[w], v, j)) v = wv[w], j = wj[w];
       if (k == 0) d0_sh = v;
       // truncation (Sec. 4): stop at the first k with R_kk < eps R_00, i.e.
       // d < eps^2 d_0.  Any positive remainder is kept otherwise, even near
@@ -154,6 +162,7 @@ __global__ void __launch_bounds__(256) k_interp_factor(const InterpTask<T>* __re
       // non-positive one ends the factorization early.
       const double floor2 = DBL_EPSILON * DBL_EPSILON;
       stop_sh = (!(v > 0.0) || v < fmax(eps * eps, floor2) * d0_sh) ? 1 : 0;
+      if (!(v < INFINITY)) *d.bad = d.p + 1;
       piv_sh = j;
       if (!stop_sh) {
         used[j] = 1;

@@ -36,15 +36,15 @@ def _nan_between_survivors(p, levels, sign):
     return pair
 
 
-@pytest.mark.parametrize("form", ["coloured", "simultaneous", "randomized"])
+@pytest.mark.parametrize("form", ["coloured", "simultaneous", "randomized", "InS", "In"])
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("dim,n,levels", [(2, 33, 3), (3, 16, 3), (3, 21, 6)])
 @pytest.mark.parametrize("sign", [1.0, -1.0])
 def test_nan_coupling_is_reported(cuda_ok, sign, dim, n, levels, precision, form):
     p = I.laplacian_2d(n) if dim == 2 else I.laplacian_3d(n)
     pair = _nan_between_survivors(p, levels, sign)
-    kw = {"compression": "randomized"} if form == "randomized" else {"sparsify_order": form}
-    s = Solver.from_problem(p, levels=levels, eps=1e-2, precision=precision, **kw)
+    option = {"randomized": "compression", "InS": "variant", "In": "variant"}.get(form, "sparsify_order")
+    s = Solver.from_problem(p, levels=levels, eps=1e-2, precision=precision, **{option: form})
     try:
         with pytest.raises(SpandError) as ei:
             s.factorize()

@@ -29,15 +29,16 @@ def _problem(dim, n, part):
 
 
 @pytest.mark.parametrize("part", ["all", "half"])
-@pytest.mark.parametrize("order", ["coloured", "simultaneous"])
+@pytest.mark.parametrize("form", ["coloured", "simultaneous", "InS", "In"])
 @pytest.mark.parametrize("precision", ["fp64", "fp32", "tf32"])
 @pytest.mark.parametrize("dim,n,levels", [(2, 33, 6), (3, 16, 4), (3, 21, 6)])
-def test_decoupled_interfaces(cuda_ok, dim, n, levels, precision, order, part):
+def test_decoupled_interfaces(cuda_ok, dim, n, levels, precision, form, part):
     import torch
     p = _problem(dim, n, part)
     b = I.rhs(p.n, 6)
     ref = sla.spsolve(p.to_scipy().tocsc(), b)
-    s = Solver.from_problem(p, levels=levels, eps=1e-3, tol=1e-12, precision=precision, sparsify_order=order)
+    s = Solver.from_problem(p, levels=levels, eps=1e-3, tol=1e-12, precision=precision,
+                            **{"variant" if form in ("InS", "In") else "sparsify_order": form})
     try:
         s.factorize()
         x, it, rr = s.solve(torch.from_numpy(b).cuda())
