@@ -154,7 +154,10 @@ struct LaGeom {
   // as many as 8 loads in flight cover (the taller ones take several rounds);
   // with LA_STREAM narrow items of 8 columns instead of wide ones: the rounds of
   // many warps overlap, and the items' fixed cost (operand loads, shuffles) is
-  // spread over more bytes.
+  // spread over more bytes.  One apply at 48^3, 64^3, 96^3 FP32, 64^3, 30^3 FP64:
+  // as here 0.279, 0.458, 0.946, 1.166, 0.265 ms; wide items with LA_STREAM too
+  // 0.297, 0.510, 1.175, 1.466, 0.281; never wide (2 from 16 VW rows on) 0.309,
+  // 0.494, 0.968, 1.238, 0.322.
   __host__ __device__ static int shape(int R, int mode) {
     return R <= 8 * VW ? 8 : R <= 16 * VW ? 4 : R <= 32 * VW || mode == LA_STREAM ? 2 : R <= 64 * VW ? -4 : R <= 128 * VW ? -2 : -1;
   }

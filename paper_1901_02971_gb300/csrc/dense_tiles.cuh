@@ -206,7 +206,8 @@ __device__ __forceinline__ void store_tile(const SqTileB<T, B>& s, T* P, int ld,
 // named barriers (bars 1, 2: rows published; 3, 4: pivot rows formed; by step
 // parity), which also alternate the buffers.  With every warp waiting for the
 // whole update and the pivot rows formed by warp 0, k_potrf_diag took 38 us on
-// average over a 64^3 factorization, now 31 (pivot family 8.4 -> 7.7 ms).  1 / U_kk comes from one reciprocal square root.  Returns false
+// average over a 64^3 factorization, now 31 (pivot family 8.4 -> 7.7 ms).
+// 1 / U_kk comes from one reciprocal square root.  Returns false
 // (for every thread) if a pivot is not positive; nothing is stored then.
 constexpr int POTRF_NT = 160;  // threads: 4 holder warps and the pivot warp
 __device__ __forceinline__ void bar_arrive(int id, int n) {

@@ -453,7 +453,8 @@ __global__ void __launch_bounds__(NT) k_trsm_cols(const TrsmTask<T>* __restrict_
 // Pull form of A_{ab} -= sum_s X_{as} X_{bs}^T over the separators s adjacent
 // to both a and b (Sec. 2.4), one 64x64 output tile per CTA, contributors in a
 // fixed order (deterministic, no atomics).  Writes block (a,b) in a's row and
-// its transpose (b,a) in b's row.
+// its transpose (b,a) in b's row.  The interpolative transforms' updates, and the
+// elimination's where the workspace of the two-launch form below is not to be had.
 template <typename T>
 __global__ void __launch_bounds__(NT) k_schur(const SchurTile* __restrict__ tiles,
                                              const SchurBlock<T>* __restrict__ blocks,

@@ -81,9 +81,30 @@ constexpr int kGramShare = 8;
 // 5.50 / 5.42 / 5.33, 64^3 TF32 37.8 / 37.7 / 37.7 / 37.5; no limit gains nothing more.
 constexpr size_t kInPlaceBytes = 65536;
 constexpr int kAuxStreams = 8;
-constexpr double kCombineWork = 2e9;      // n^2 m of a step's separators up to which their G blocks are formed (FP32)
-constexpr double kApplyStreamBytes = 2e7;  // factor bytes of a phase of the apply from which it is LA_STREAM
-constexpr int64_t kApplyFewItems = 2000;    // 8-row items up to which it is LA_FEW
+// Where the apply's phases are cut (apply_levels.cuh).  Milliseconds of one
+// spand_apply call, diffusion problems of 48^3, 64^3, 96^3 and 290^2 unknowns
+// (FP32), then 64^3, 30^3 and 64^2 (FP64).
+//
+// n^2 m of a step's separators up to which their G blocks are formed, FP32 and
+// FP64 (whose products cost more).  FP32 at 0 / 2e8 / 2e9 / 2e10 / no limit:
+// 0.323 / .279 / .279 / .266 / .266, .512 / .462 / .461 / .433 / .432, 1.024 /
+// .952 / .948 / .947 / .899, .275 / .231 / .231 / .231 / .230; beyond 2e9 these are
+// the leaves' G, which cost a factorization 0.3, 0.8 and 2.5 ms at 48^3, 64^3, 96^3
+// and double the leaves' factor.  FP64 at 0 / 5e6 / 1e8 / 2e9 / no limit: 1.212 /
+// 1.212 / 1.164 / 1.149 / 1.144, .320 / .300 / .265 / .259 / .260, .218 / .171 from
+// 5e6 on; the factorization of 64^3 takes 0.7 ms more at 1e8, 3.2 at 2e9, 23 with
+// all, that of 30^3 0.3, 0.8 and 1.2.
+constexpr double kCombineWork = 2e9, kCombineWork64 = 1e8;
+// Factor bytes of a phase from which it is LA_STREAM.  At 0 / 2e6 / 2e7 / 1e8 / no
+// phase: .329 / .308 / .277 / .279 / .302, .515 / .486 / .461 / .461 / .521, 1.008 /
+// .977 / .946 / 1.001 / 1.281, .224 / .227 / .231 / .231 / .231; FP64 1.289 / 1.220 /
+// 1.166 / 1.221 / 1.475, .325 / .267 / .269 / .284 / .284, .171 throughout.
+constexpr double kApplyStreamBytes = 2e7;
+// 8-row items up to which it is LA_FEW.  At 0 / 500 / 2000 / 8000 / no limit: .287 /
+// .279 / .278 / .278 / .279, .469 / .463 / .461 / .466 / .467, .955 / .949 / .947 /
+// .952 / .954, .231 throughout; FP64 1.211 / 1.171 / 1.167 / 1.203 / 1.205, .267 /
+// .256 / .268 / .268 / .269, .171 throughout.
+constexpr int64_t kApplyFewItems = 2000;
 constexpr int kApplyCtasPerSm = 4;  // the most CTAs per SM the apply autotuner tries
 // Phases per launch of the apply at most (their descriptors take 72 KB of shared memory, three CTAs per SM).
 constexpr int kLevelMaxPhases = 96;
@@ -513,7 +534,7 @@ struct spand_handle_s {
   PinnedStage stage;  // host side of every descriptor upload of a factorization
   DevBuf scratch[2];
   DevBuf d_vals, d_asm_row, d_asm_off, d_prow, d_pcol, d_pval, d_pval_src, d_perm;
-  DevBuf d_vec, d_tmp, d_save, d_bin, d_bout;
+  DevBuf d_vec, d_tmp, d_save;
   DevBuf d_piv64;  // FP64 copies of the pivot blocks of FP32 factors (scratch)
   DevBuf d_rand;   // sketches, products and state of the randomized compression (scratch)
   DevBuf d_interp; // Gram matrices, R rows and pivot orders of the interpolative variants (scratch)
@@ -1850,7 +1871,8 @@ static void add_level_step(spand_handle h, LevelProgram<T>& lp, int t, const std
   }
   typename LevelProgram<T>::Step st;
   st.combined = !gfac.empty();
-  {  // LA_STREAM by bytes; LA_FEW by the 8-row items of the forward phases, where those take several rounds of loads
+  {  // LA_STREAM by bytes; LA_FEW by the 8-row items of the forward phases, where those take several rounds of
+     // loads (without that condition 30^3 FP64 0.265 -> 0.300 ms, 64^2 FP64 0.172 -> 0.185, FP32 unchanged)
     const int round = 64 * LaGeom<T>::VW / 2;  // columns that 8 loads of an 8-row item cover
     double eb = 0, sb = 0;
     int64_t ei = 0, si = 0;
@@ -2519,7 +2541,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
     if (levels) {
       double work = 0;
       for (int i : seps) work += (double)sz[i] * sz[i] * (lay.W[i] - sz[i]);
-      if (!h->lean && work <= kCombineWork / (sizeof(T) == 8 ? 20 : 1)) {
+      if (!h->lean && work <= (sizeof(T) == 8 ? kCombineWork64 : kCombineWork)) {
         gfac.assign(n, nullptr);
         std::vector<CombineTask<T>> gt;
         for (int i : seps) {
@@ -2722,7 +2744,7 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
       std::vector<int> treg;    // lane-group size of the register-resident kernel (0: chunked kernel)
       const int ncol = st.ncolours();
       size_t wbytes = 0, qbytes = 0;
-      struct WOff { size_t nrm, v, tau, qc, gw; };
+      struct WOff { size_t v, tau, qc, gw; };
       std::vector<WOff> woff;
       const size_t CB = kCpqrChunkBudget;
       const int max_cluster = kCpqrMaxCluster;
@@ -2772,7 +2794,6 @@ static int factorize_impl(spand_handle h, cudaStream_t s) {
                                                 std::to_string(mm) + " columns)"};
         const bool resident = res_smem(C) <= CB;
         WOff w;
-        w.nrm = 0;
         w.v = qbytes; qbytes += align256((size_t)sz[p] * sz[p] * sizeof(T));
         w.tau = qbytes; qbytes += align256((size_t)sz[p] * sizeof(T));
         w.qc = qbytes; qbytes += align256((size_t)sz[p] * sz[p] * sizeof(T));
