@@ -206,7 +206,7 @@ HBM_BOUND = {"copy", "apply", "pcg"}
 # of one factorization or solve), with the SHA-256 of the kernel source the
 # counters were taken on: a changed kernel reports null until re-measured.
 # The capture and its command are summarised under profiles/ (DRAM traffic, 64^3).
-CPQR_DRAM_BYTES = 580.39e6 + 6.00e6  # read + written by the 205 launches of one factorization
+CPQR_DRAM_BYTES = 580.04e6 + 6.24e6  # read + written by the 205 launches of one factorization
 MEASURED_TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum: "cpqr", of all the
     # sparsification launches of one factorization (k_cpqr_cluster,
@@ -215,10 +215,10 @@ MEASURED_TRAFFIC = {
     # one pass
     "cpqr": {"bytes_per_step": CPQR_DRAM_BYTES,
              "src": ["paper_1901_02971_gb300/csrc/cpqr_cluster.cuh", "paper_1901_02971_gb300/csrc/cpqr_reg.cuh"],
-             "sha256": ["608d408ffc825989804794082c47f2be26bd40604cf0628e30b24e3a884a8808",
-                        "f4375f2638107797fe808912ff23db71eba06329efe4f946106ee94aebe58cd8"]},
-    "apply": {"bytes_per_launch": (3051.0e6 + 63.2e6) / 3, "src": "paper_1901_02971_gb300/csrc/apply_levels.cuh",
-              "sha256": "866a25c4f6ad6a73ba0d2cea6f86a869de486d75afca718475ab68bc7e775ab5"},
+             "sha256": ["2d0179ec68664375a91ce5d7cccf4ae4bc8bbbd6c1d2f6ab64dda2135e6518df",
+                        "a2bd4bd6eee48d9d59de68a625e6487fe2bff8efe92f32390adcdafd95b64296"]},
+    "apply": {"bytes_per_launch": (3050.8e6 + 62.8e6) / 3, "src": "paper_1901_02971_gb300/csrc/apply_levels.cuh",
+              "sha256": "c85e6d6f1f972f6b3432de39f013a27abcf164c8f8f630acdb5260c4f6331584"},
 }
 
 
