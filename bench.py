@@ -206,7 +206,7 @@ HBM_BOUND = {"copy", "apply", "pcg"}
 # of one factorization or solve), with the SHA-256 of the kernel source the
 # counters were taken on: a changed kernel reports null until re-measured.
 # The capture and its command are summarised under profiles/ (DRAM traffic, 64^3).
-CPQR_DRAM_BYTES = 580.04e6 + 6.24e6  # read + written by the 205 launches of one factorization
+CPQR_DRAM_BYTES = 580.11e6 + 6.23e6  # read + written by the 205 launches of one factorization
 MEASURED_TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum: "cpqr", of all the
     # sparsification launches of one factorization (k_cpqr_cluster,
@@ -215,7 +215,7 @@ MEASURED_TRAFFIC = {
     # one pass
     "cpqr": {"bytes_per_step": CPQR_DRAM_BYTES,
              "src": ["paper_1901_02971_gb300/csrc/cpqr_cluster.cuh", "paper_1901_02971_gb300/csrc/cpqr_reg.cuh"],
-             "sha256": ["2d0179ec68664375a91ce5d7cccf4ae4bc8bbbd6c1d2f6ab64dda2135e6518df",
+             "sha256": ["063616e61f53016735fc6184f3a493e54ffeb4433f49c25f69a66b7ff8af6e1f",
                         "a2bd4bd6eee48d9d59de68a625e6487fe2bff8efe92f32390adcdafd95b64296"]},
     "apply": {"bytes_per_launch": (3050.8e6 + 62.8e6) / 3, "src": "paper_1901_02971_gb300/csrc/apply_levels.cuh",
               "sha256": "c85e6d6f1f972f6b3432de39f013a27abcf164c8f8f630acdb5260c4f6331584"},

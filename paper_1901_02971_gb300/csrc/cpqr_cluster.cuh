@@ -677,8 +677,8 @@ __global__ void __launch_bounds__(NT) k_cpqr_cluster(const CpqrTask<T>* __restri
 // sparsification's critical path.  Block b of
 // an interface (nb blocks each) takes the column pairs (c, c + nb NW) with
 // c = b NW + warp (mod 2 nb NW), so every block meets chains of every length;
-// V is copied into shared memory when it fits beside the rank's tau, which
-// always does (smem_elems elements in all).
+// up to 512 rows tau is kept in shared memory, and V where it fits beside it
+// (smem_elems elements in all, room for np entries of tau at least).
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT) k_form_q(const CpqrTask<T>* __restrict__ tasks,
                                                  const int32_t* __restrict__ list,
@@ -692,25 +692,26 @@ __global__ void __launch_bounds__(NT) k_form_q(const CpqrTask<T>* __restrict__ t
   T* tau_s = reinterpret_cast<T*>(smraw);
   T* vs = tau_s + cq_al16((size_t)r * sizeof(T)) / sizeof(T);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int k = tid; k < r; k += NT) tau_s[k] = d.tau[k];
-  const T* Vsrc = d.V;
-  const size_t nv = (size_t)np * r;
-  if (np <= 32 * 16 && (size_t)(vs - tau_s) + nv <= (size_t)smem_elems) {
-    for (size_t e = tid; e < nv; e += NT) vs[e] = __ldcg(d.V + e);  // rows < k of column k are never read
-    Vsrc = vs;
-  }
-  __syncthreads();
   if (np <= 32 * 16) {
+    for (int k = tid; k < r; k += NT) tau_s[k] = d.tau[k];
+    const T* Vsrc = d.V;
+    const size_t nv = (size_t)np * r;
+    if ((size_t)(vs - tau_s) + nv <= (size_t)smem_elems) {
+      for (size_t e = tid; e < nv; e += NT) vs[e] = __ldcg(d.V + e);  // rows < k of column k are never read
+      Vsrc = vs;
+    }
+    __syncthreads();
     cq_form_q_any<T>(d, Vsrc, tau_s, r, np, b, nb);
     return;
   }
-  // tall interfaces: one warp per column, V and the column in global memory
+  // tall interfaces: one warp per column, V, tau and the column in global memory
+  // (a rank of any size: nothing of it is kept in shared memory)
   for (int c = b * NW + warp; c < r; c += nb * NW) {
     T* col = d.Qc + (size_t)c * np;
     for (int i = lane; i < np; i += 32) col[i] = (i == c) ? T(1) : T(0);
     __syncwarp();
     for (int k = c; k >= 0; --k) {
-      const T tk = tau_s[k];
+      const T tk = __ldcg(d.tau + k);
       if (tk == T(0)) continue;
       const T* v = d.V + (size_t)k * np;
       T w = 0;

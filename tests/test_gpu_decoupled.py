@@ -80,3 +80,23 @@ def test_decoupled_interfaces_randomized(cuda_ok, dim, n, levels, precision, par
                         sketch=lambda t, c, m, ell: O.sketch_philox(0, t, c, m, ell))
         for t in range(1, levels + 1):
             assert np.array_equal(ranks[t - 1], F.sizes_after[t - 1]), t
+
+
+@pytest.mark.parametrize("part", ["all", "half"])
+def test_tall_interfaces(cuda_ok, part):
+    """Interfaces of 578 dofs, beyond the 512 that the basis kernel holds in
+    registers, with and without columns to be compressed against."""
+    import torch
+    p = _problem(3, 34, part)
+    s = Solver.from_problem(p, levels=3, eps=1e-3, tol=1e-12, precision="fp32")
+    try:
+        s.factorize()
+        before, after = s.ranks(1)
+        tall = np.asarray(before)[np.asarray(s.step(1)["elim"]) == 0].max()
+        assert tall > 512
+        if part == "all":
+            assert np.asarray(after).max() == tall  # kept whole
+        x, it, rr = s.solve(torch.from_numpy(I.rhs(p.n, 6)).cuda())
+    finally:
+        s.close()
+    assert rr <= 1e-12 and it <= (3 if part == "all" else 20)
